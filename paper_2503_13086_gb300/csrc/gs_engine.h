@@ -129,7 +129,8 @@ struct Raster {
   gs_status upload(cudaStream_t s);
   void mark(cudaStream_t s, int k);
   gs_status enqueue_forward_head(cudaStream_t s, const float* params, int stride_, bool size_exactly);
-  gs_status enqueue_forward_tail(cudaStream_t s, float* image, float* T, unsigned* last, unsigned* gp);
+  // tile_flags: the loss that follows starts on finished tiles (enqueue_loss with after_forward)
+  gs_status enqueue_forward_tail(cudaStream_t s, float* image, float* T, unsigned* last, unsigned* gp, bool tile_flags);
   // after_forward: the loss follows this step's blend forward directly in the stream (its blocks then
   // start as the forward completes the tiles under them)
   void enqueue_loss(cudaStream_t s, const float* image, float* dimage, bool after_forward);

@@ -557,7 +557,7 @@ struct Field {
     R.upload(stream);
     if ((s = R.enqueue_forward_head(stream, static_cast<float*>(params.p), stride, size_exactly))) return s;
     if ((s = R.enqueue_forward_tail(stream, static_cast<float*>(step_img.p), static_cast<float*>(step_T.p),
-                                    static_cast<unsigned*>(step_last.p), static_cast<unsigned*>(step_gp.p))))
+                                    static_cast<unsigned*>(step_last.p), static_cast<unsigned*>(step_gp.p), true)))
       return s;
     R.enqueue_loss(stream, static_cast<float*>(step_img.p), static_cast<float*>(step_dimg.p), true);
     R.enqueue_backward(stream, static_cast<float*>(params.p), static_cast<float*>(step_img.p),
@@ -736,7 +736,7 @@ struct Field {
         if (cs == GS_ERR_OOM || cs == GS_ERR_BUDGET || cs == GS_ERR_CAPACITY) break;
         if ((s = cs)) break;
         if ((s = R.enqueue_forward_tail(stream, img, static_cast<float*>(step_T.p), static_cast<unsigned*>(step_last.p),
-                                        static_cast<unsigned*>(step_gp.p))))
+                                        static_cast<unsigned*>(step_gp.p), true)))
           break;
         R.enqueue_loss(stream, img, dimg, true);
         R.enqueue_backward(stream, static_cast<float*>(params.p), img, static_cast<unsigned*>(step_last.p), dimg,
@@ -1446,7 +1446,7 @@ gs_status gs_render(gs_field* ff, const gs_camera* cam, float* out_rgb, float* o
   R.reset_ledger(f->stream);
   R.upload(f->stream);
   if ((s = R.enqueue_forward_head(f->stream, static_cast<float*>(f->params.p), f->stride, true))) return s;
-  if ((s = R.enqueue_forward_tail(f->stream, out_rgb, out_T, static_cast<unsigned*>(f->step_last.p), nullptr))) return s;
+  if ((s = R.enqueue_forward_tail(f->stream, out_rgb, out_T, static_cast<unsigned*>(f->step_last.p), nullptr, false))) return s;
   f->sized_for_views = false;
   R.enqueue_readback(f->stream);
   cudaError_t e = cudaStreamSynchronize(f->stream);

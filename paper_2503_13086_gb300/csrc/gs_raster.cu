@@ -361,7 +361,8 @@ gs_status Raster::enqueue_forward_head(cudaStream_t s, const float* params, int 
   return GS_OK;
 }
 
-gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, unsigned* last, unsigned* gp) {
+gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, unsigned* last, unsigned* gp,
+                                       bool tile_flags) {
   last_gp = gp;
   if (zeroB_pending) cudaMemsetAsync(zeroB.p, 0, zeroB_bytes, s);
   zeroB_pending = false;
@@ -383,8 +384,8 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
   mark(s, 5);
   launch_blend_forward(tiling, vd(), n_views, n_tiles, ranges(), v0, proj(), sp(), ctl(),
                        static_cast<const int*>(order.p), image, T, last, gp, static_cast<float4*>(ckpt.p),
-                       static_cast<unsigned*>(cmask.p), chunk_tile(), static_cast<int*>(tile_chunks.p), tile_done(),
-                       num_sms, s);
+                       static_cast<unsigned*>(cmask.p), chunk_tile(), static_cast<int*>(tile_chunks.p),
+                       tile_flags ? tile_done() : nullptr, num_sms, s);
   mark(s, 6);
   return GS_OK;
 }
@@ -501,7 +502,7 @@ gs_status gs_raster_forward(gs_raster* rr, void* stream, const float* params, in
   r->upload(s);
   if ((st = r->enqueue_forward_head(s, params, (int)stride, true))) return st;
   if ((st = r->ensure_instances(r->m_cap))) return st;
-  if ((st = r->enqueue_forward_tail(s, out_image, out_T, out_last, out_gp))) return st;
+  if ((st = r->enqueue_forward_tail(s, out_image, out_T, out_last, out_gp, false))) return st;
   r->have_forward = true;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("forward launch: ") + cudaGetErrorString(e));

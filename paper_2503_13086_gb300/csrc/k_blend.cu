@@ -12,10 +12,19 @@
 // and publishes it on an mbarrier, so staging overlaps the other warps' walk and a fast warp can run
 // a job ahead of the tile's slowest block instead of waiting for it at a CTA barrier.  Jobs are
 // walked in chunks of 32.  A warp skips a Gaussian outright when the bounding box of its 1/255 cutoff
-// ellipse misses the warp's block (warp-uniform); for the others each pixel tests its exponent
-// against -ln(255 opacity) and only then evaluates exp, alpha, the early stop and the blending.  (A
-// separate, pipelined candidate pass before the sequential walk computed the exponent twice for
-// every candidate: equal on sparse views, 6-10 % slower on dense ones.)
+// ellipse misses the warp's block (warp-uniform).  The others are taken two at a time without a branch:
+// every lane evaluates both exponents and alphas, then blends them in list order under predicates.  A
+// pixel's walk is one dependent chain, and the longest lists set the kernel's duration from a few
+// thousand Gaussians up, so what counts is the chain's length per candidate: with a branch per test
+// (cutoff, alpha, stop) it was about 300 cycles, in this form about 210 when a CTA has its SM to itself,
+// and about 48 instead of 62 instructions.  A stopped pixel's x becomes NaN, which fails every later
+// test by itself; the last index and G_p follow from the chunk's mask.  Measured: 54 -> 32 us on a
+// 128 x 97 view of 3,400 Gaussians, 54 -> 39 us at 640 x 361 (20k), 120 -> 108 us at 1297 x 840 (200k,
+// 32M blended pairs), 440 -> 345 us at 1.9M, 856 -> 755 us for nine views of 500k.  (A lone last candidate
+// is evaluated alone: evaluating it twice cost 4 % on the nine views.)  Measured and not kept: two
+// lanes per pixel, each with its own candidate, on 4 x 4 blocks (the blending is then done by both:
+// 183 us at 200k); the next pair's records read during the blending (124 us); 80 registers and three
+// CTAs per SM (291 us at 1.9M, but 843 us on the nine views); a staging warp of its own (139 us).
 // Per (pixel, chunk) K6 stores the transmittance and colour at the chunk start and a 32-bit mask
 // of the Gaussians actually blended; a tile gets no more batches once every warp's pixels stopped.
 // When the last of a tile's warps leaves it, the tile is flagged complete (a GPU-scope release), so
@@ -305,20 +314,28 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
   bool ok = warp != 0 || stage(0);
 
   // this thread's pixel of the current tile
-  int my_seq = -1;
-  long long my_t = 0;
-  long long pix_base = 0;
-  int px = 0, py = 0, Wv = 0;
-  long long HWv = 0, cb = 0;
-  bool inside = false, done = true, counted = true;
+  int my_seq = -1, my_t = 0, my_v = 0;
+  long long my_chunk = 0;  // chunk 0's slot of this pixel in the checkpoints and masks
+  bool counted = true;
   float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
   unsigned last = 0u, gp = 0u, neval = 0u;
-  float pxf = 0.f, pyf = 0.f;
+  float pxf = 0.f, pyf = 0.f;  // pxf is NaN where there is no pixel or it has stopped
+  auto pixel = [&](int& px, int& py) {
+    const ViewDev& V = views[my_v];
+    const int local = (int)(my_t - V.tile_base);
+    int ox, oy;
+    S::slot_xy(tid, ox, oy);
+    px = local % V.gx * TW + ox;
+    py = local / V.gx * TH + oy;
+  };
   // (warp-uniform: every lane of the warp leaves the tile at the same job)
   auto finish_tile = [&]() {
     if (my_seq < 0) return;
-    if (inside) {
-      const long long pix = (long long)py * Wv + px;
+    const ViewDev& V = views[my_v];
+    int px, py;
+    pixel(px, py);
+    if (px < V.W && py < V.H) {
+      const long long pix = (long long)py * V.W + px, HWv = (long long)V.W * V.H, pix_base = V.pix_base;
       float* img = image + 3 * pix_base;
       img[pix] = C0 + T * bg0;
       img[HWv + pix] = C1 + T * bg1;
@@ -340,6 +357,8 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
     // every pixel of the tile (the loss forward starts a block once the tiles under it are flagged).
     // Job j + 1 is staged only once every warp is through job j - 1, so the warps that have not left
     // a tile are on the tiles of three consecutive jobs at most: four counters are never shared.
+    // (Without tile flags nothing reads this grid's output before it has completed.)
+    if (!tile_done) return;
     __syncwarp();
     if (lane == 0) {
       unsigned* fin = &s_fin[my_seq & 3];
@@ -350,6 +369,45 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
         red_release_add_u32(tile_done + my_t, 1u);
       }
     }
+  };
+
+  struct Cand {
+    float alpha, r, g, b;
+    bool use;
+  };
+  // Alpha of entry q of buffer `buf` at this pixel, and whether the pixel takes it (before its stop
+  // test).  A pixel that has stopped (or lies outside the image) has pxf = NaN, so that no comparison
+  // of its exponent holds.
+  auto eval = [&](int buf, int q) -> Cand {
+    const float2 xy = *reinterpret_cast<const float2*>(&s_xyo[buf][q]);
+    const float4 co = s_con[buf][q];
+    const float4 c = s_rgb[buf][q];
+    const float power = splat_power(co.x, co.y, co.z, __fsub_rn(xy.x, pxf), __fsub_rn(xy.y, pyf));
+    Cand e;
+    e.alpha = fminf(kAlphaMax, __fmul_rn(c.w, splat_exp(power)));
+    e.use = power <= 0.f && power >= co.w && e.alpha >= kAlphaMin;
+    e.r = c.x;
+    e.g = c.y;
+    e.b = c.z;
+    return e;
+  };
+  // Blends a candidate the pixel takes; true when the pixel stops at it.
+  auto blend = [&](const Cand& e, bool use, unsigned bit, int jg, unsigned& mask) -> bool {
+    const float testT = __fmul_rn(T, __fsub_rn(1.f, e.alpha));
+    const bool stop = use && testT < kTransMin;
+    if (stop) {
+      pxf = __int_as_float(0x7fffffff);
+      neval = (unsigned)jg + 1u;
+    }
+    if (use && !stop) {
+      const float w = __fmul_rn(e.alpha, T);
+      C0 = __fmaf_rn(e.r, w, C0);
+      C1 = __fmaf_rn(e.g, w, C1);
+      C2 = __fmaf_rn(e.b, w, C2);
+      T = testT;
+      mask |= bit;
+    }
+    return stop;
   };
 
   for (int j = 0; ok; ++j) {
@@ -363,73 +421,60 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
       finish_tile();
       if (jb.end) break;
       my_seq = jb.seq;
-      my_t = jb.t;
-      const int v = view_of_tile(views, n_views, jb.t);
-      const ViewDev& V = views[v];
-      const long long local = jb.t - V.tile_base;
-      const int tx = (int)(local % V.gx), ty = (int)(local / V.gx);
-      int ox, oy;
-      S::slot_xy(tid, ox, oy);
-      px = tx * TW + ox;
-      py = ty * TH + oy;
-      Wv = V.W;
-      HWv = (long long)V.W * V.H;
-      pix_base = V.pix_base;
-      inside = px < V.W && py < V.H;
-      pxf = (float)px;
+      my_t = (int)jb.t;
+      my_v = view_of_tile(views, n_views, jb.t);
+      int px, py;
+      pixel(px, py);
+      pxf = px < views[my_v].W && py < views[my_v].H ? (float)px : __int_as_float(0x7fffffff);
       pyf = (float)py;
-      cb = chunk_base(jb.start, jb.t);
+      my_chunk = chunk_base(jb.start, jb.t) * kPix + tid;
       T = 1.f;
       C0 = C1 = C2 = 0.f;
       last = gp = 0u;
       neval = (unsigned)jb.L;
-      done = !inside;
       counted = false;
     }
     // walk this job's chunks (a warp whose pixels have all stopped still records empty masks)
     const int nb = min(BATCH, jb.L - jb.b0);
     for (int c0 = 0; c0 < nb; c0 += kChunk) {
       const int jg0 = jb.b0 + c0;
-      const long long chunk = cb + (jg0 >> 5);
+      const long long at = my_chunk + (long long)(jg0 >> 5) * kPix;
       const int ce = min(kChunk, nb - c0);
       // entries of this chunk whose cutoff box reaches this warp's block (warp-uniform)
-      const unsigned rel = __ballot_sync(0xffffffffu, lane < ce && ((s_bm[buf][c0 + lane] >> warp) & 1u));
-      if (done) {
-        cmask[chunk * kPix + tid] = 0u;
+      unsigned cand = __ballot_sync(0xffffffffu, lane < ce && ((s_bm[buf][c0 + lane] >> warp) & 1u));
+      const bool done = pxf != pxf;
+      if (__all_sync(0xffffffffu, done)) {
+        cmask[at] = 0u;
         continue;
       }
-      if (jg0 > 0) ckpt[chunk * kPix + tid] = make_float4(T, C0, C1, C2);
-      unsigned cand = rel;
+      if (jg0 > 0 && !done) ckpt[at] = make_float4(T, C0, C1, C2);
       unsigned mask = 0u;
+      // One straight line per candidate, two candidates in flight: every lane evaluates both
+      // exponents and alphas, then they are blended in list order under predicates.
       while (cand) {
-        const int q = __ffs(cand) - 1;
-        cand &= cand - 1u;
-        const float4 xy = s_xyo[buf][c0 + q];
-        const float4 co = s_con[buf][c0 + q];
-        const float power = splat_power(co.x, co.y, co.z, __fsub_rn(xy.x, pxf), __fsub_rn(xy.y, pyf));
-        if (power > 0.f || !(power >= co.w)) continue;
-        const float4 c = s_rgb[buf][c0 + q];
-        const float alpha = fminf(kAlphaMax, __fmul_rn(c.w, splat_exp(power)));
-        if (alpha < kAlphaMin) continue;
-        const float testT = __fmul_rn(T, __fsub_rn(1.f, alpha));
-        if (testT < kTransMin) {
-          done = true;
-          neval = (unsigned)(jg0 + q) + 1u;
+        const unsigned bit0 = cand & (0u - cand);
+        const int q0 = 31 - __clz(bit0);
+        cand ^= bit0;
+        if (!cand) {
+          const Cand e0 = eval(buf, c0 + q0);
+          blend(e0, e0.use, bit0, jg0 + q0, mask);
           break;
         }
-        const float w = __fmul_rn(alpha, T);
-        C0 = __fmaf_rn(c.x, w, C0);
-        C1 = __fmaf_rn(c.y, w, C1);
-        C2 = __fmaf_rn(c.z, w, C2);
-        T = testT;
-        last = (unsigned)(jg0 + q) + 1u;
-        ++gp;
-        mask |= 1u << q;
+        const unsigned bit1 = cand & (0u - cand);
+        const int q1 = 31 - __clz(bit1);
+        cand ^= bit1;
+        const Cand e0 = eval(buf, c0 + q0), e1 = eval(buf, c0 + q1);
+        const bool stop = blend(e0, e0.use, bit0, jg0 + q0, mask);
+        blend(e1, e1.use && !stop, bit1, jg0 + q1, mask);
       }
-      cmask[chunk * kPix + tid] = mask;
+      if (mask) {
+        last = (unsigned)(jg0 + 32 - __clz(mask));
+        gp += __popc(mask);
+      }
+      cmask[at] = mask;
     }
     // this warp's pixels have all stopped: the stager need not stage more of the tile for it
-    if (!counted && __all_sync(0xffffffffu, done)) {
+    if (!counted && __all_sync(0xffffffffu, pxf != pxf)) {
       counted = true;
       if (lane == 0) atomicSub(&s_live[my_seq % kFwdBufs], 1);
     }

@@ -1,0 +1,80 @@
+"""The blend forward's candidate walk at the list lengths where it changes shape: pairs and a lone last
+candidate, whole and partial chunks of 32, one and several staged batches, pixels that stop early and
+pixels outside the image.  One 16 x 16 tile, isotropic Gaussians; the reference blends the kernel's own
+records front to back in float64.
+
+Tolerance, derived: an isotropic conic's exponent terms share a sign, so its rounding is at most
+4 u x 5.55 (u = 2^-24, the exponent's range is [-ln 255, 0]) = 1.3e-6; the exponential instruction adds
+2^-22 and the rounding of its argument (at most 8 u ln 2), together 2.0e-6 relative on alpha.  A pixel's
+transmittance carries sum alpha / (1 - alpha) <= 10 of those (it stops at 1e-4) and 2 u per factor, the
+colour one more and u per sum: for 600 entries at most 11 x 2.0e-6 + 600 x 3 x 6e-8 = 1.3e-4 of the
+colour scale, and the colours here are below 0.75: 1e-4.  Pixels where a decision (alpha against 1/255, T
+against 1e-4) is closer than its own error are left out of the comparison of the counts."""
+import numpy as np
+import pytest
+
+import gsinputs as gi
+from helpers import gpu_forward
+
+pytestmark = pytest.mark.gpu
+
+
+def _scene(n, opacity, seed):
+    rng = np.random.default_rng(seed)
+    p = np.zeros((59, (n + 31) // 32 * 32), np.float32)
+    p[0:2, :n] = rng.uniform(-1.3, 1.3, (2, n))
+    p[2, :n] = rng.uniform(2.9, 3.1, n)
+    p[3:6, :n] = rng.uniform(-2.2, -1.0, n)
+    p[6, :n] = 1.0
+    p[10, :n] = np.log(opacity / (1 - opacity))
+    p[11:14, :n] = rng.uniform(-1.5, 0.8, (3, n))
+    return p
+
+
+def _blend64(g, w, h):
+    order = g["vals"].astype(np.int64)
+    m, con, rgb, op = (g["rec"][k][order].astype(np.float64) for k in ("mean2d", "conic", "rgb", "opacity"))
+    py, px = np.mgrid[0:h, 0:w].astype(np.float64)
+    T = np.ones((h, w))
+    C = np.zeros((3, h, w))
+    last, gp = np.zeros((h, w), np.int64), np.zeros((h, w), np.int64)
+    neval = np.full((h, w), len(order))
+    done, clear = np.zeros((h, w), bool), np.ones((h, w), bool)
+    for k in range(len(order)):
+        dx, dy = m[k, 0] - px, m[k, 1] - py
+        power = -0.5 * (con[k, 0] * dx * dx + con[k, 2] * dy * dy) - con[k, 1] * dx * dy
+        alpha = np.minimum(0.99, op[k] * np.exp(power))
+        clear &= done | (np.abs(alpha * 255 - 1) > 1e-5)
+        use = ~done & (power <= 0) & (alpha >= 1 / 255)
+        test = T * (1 - alpha)
+        clear &= ~use | (np.abs(test / 1e-4 - 1) > 1e-3)
+        stop = use & (test < 1e-4)
+        neval[stop] = k + 1
+        done |= stop
+        use &= ~stop
+        C += np.where(use, alpha * T, 0.0) * rgb[k][:, None, None]
+        T = np.where(use, test, T)
+        last[use] = k + 1
+        gp += use
+    return C, T, last, gp, neval, clear
+
+
+@pytest.mark.parametrize("size", [(16, 16), (13, 9)])
+@pytest.mark.parametrize("opacity", [0.03, 0.9])
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 32, 33, 255, 256, 257, 545])
+def test_walk_edges(n, opacity, size):
+    import paper_2503_13086_gb300 as gs
+    w, h = size
+    ras = gs.Raster()
+    g = gpu_forward(ras, _scene(n, opacity, 40 + n), n, [gi.identity_camera(w, h, 16.0)])
+    assert len(g["vals"]) >= 1
+    C, T, last, gp, neval, clear = _blend64(g, w, h)
+    out = g["out"]
+    assert np.abs(out["image"].cpu().numpy().reshape(3, h, w) - C)[:, clear].max() <= 1e-4
+    assert np.abs(out["T"].cpu().numpy().reshape(h, w) - T)[clear].max() <= 1.3e-4
+    assert np.array_equal(out["last"].cpu().numpy().reshape(h, w)[clear], last[clear])
+    assert np.array_equal(out["gp"].cpu().numpy().reshape(h, w)[clear], gp[clear])
+    assert clear.mean() > 0.8
+    if clear.all():
+        assert out["pairs"] == int(neval.sum())
+    ras.close()
