@@ -72,11 +72,12 @@ void launch_blend_forward(const Tiling& tl, const ViewDev* views, int n_views, l
                           cudaStream_t s);
 // Warps the blend forward launches for this problem (each adds 1 to Control::fwd_done at its end).
 long long forward_warps(const Tiling& tl, long long n_tiles, int num_sms);
+// load: the load term's gradient is added (needs gp, the forward's G_p).
 void launch_blend_backward(const Tiling& tl, const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
                            const unsigned* vals, const ProjBuffers& pb, Control* ctl, const float* image,
                            const float* dimage, const float4* ckpt, const unsigned* cmask, const int* chunk_tile,
-                           const int* tile_chunks, float4* ginst, const unsigned* gp, const StepParams* sp,
-                           int num_sms, cudaStream_t s);
+                           const int* tile_chunks, float4* ginst, const unsigned* gp, bool load, const StepParams* sp,
+                           long long m_cap, int num_sms, cudaStream_t s);
 
 // Field update (Sec. IV-B): the registered sparse points, hashed by cubic cells.
 constexpr float kCoarseCells = 4.f;  // coarse grid cell edge in fine cells (3-NN search)

@@ -400,8 +400,8 @@ void Raster::enqueue_loss(cudaStream_t s, const float* image, float* dimage, boo
 void Raster::enqueue_blend_backward(cudaStream_t s, const float* image, const float* dimage) {
   launch_blend_backward(tiling, vd(), n_views, n_tiles, ranges(), static_cast<unsigned*>(vals0.p), proj(),
                         ctl(), image, dimage, static_cast<float4*>(ckpt.p), static_cast<unsigned*>(cmask.p),
-                        chunk_tile(), static_cast<int*>(tile_chunks.p), static_cast<float4*>(ginst.p), last_gp, sp(),
-                        num_sms, s);
+                        chunk_tile(), static_cast<int*>(tile_chunks.p), static_cast<float4*>(ginst.p), last_gp,
+                        last_gp != nullptr && sp_h->lambda_load > 0.f, sp(), (long long)m_cap, num_sms, s);
   mark(s, 8);
 }
 

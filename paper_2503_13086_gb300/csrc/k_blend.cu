@@ -44,7 +44,15 @@
 // lanes through shared memory in a fixed order and added to the Gaussians' running sums.  A round's pixels share
 // few Gaussians (about 9 of 32), each blended by many of them, so this keeps more lanes busy than
 // one lane per Gaussian.  No atomics: the gradient is deterministic, and each instance's gradient
-// is written once, to its own slot.
+// is written once, to its own slot.  K8 is bound by issue (66 % at 16 warps per SM; 240 instructions per
+// Gaussian and round, of which 1.4 pair bodies are about 95) and, with few items, by one warp's latency
+// (5 cycles per instruction).  The load term is a template flag (its test and weights cost 4 registers
+// and an instruction per pair), the reciprocal of 1 - alpha the bare instruction, the conic terms' factors
+// are applied once per row sum, and the tile's position takes 32-bit divisions: 1269 -> 1221 us for nine
+// views of 500k Gaussians, 152 -> 144 at 1297 x 840 (200k), 48 -> 45 at 640 x 361 (20k), the same bits.
+// Measured and not kept: the records held twice in shared memory for the packed operands (16 bytes more
+// per Gaussian through a half-busy pipe: 163 us at 200k), the next item claimed one ahead (63 us at 20k),
+// both pairs evaluated without a branch (1323 us on the nine views, no shorter for a lone warp).
 #include "gs_device.cuh"
 #include "gs_engine.h"
 
@@ -250,8 +258,8 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
       }
       const int v = view_of_tile(views, n_views, jb.t);
       const ViewDev& V = views[v];
-      const long long local = jb.t - V.tile_base;
-      const float tx0 = (float)((int)(local % V.gx) * TW), ty0 = (float)((int)(local / V.gx) * TH);
+      const int local = (int)(jb.t - V.tile_base);
+      const float tx0 = (float)(local % V.gx * TW), ty0 = (float)(local / V.gx * TH);
       const int nb = min(BATCH, jb.L - jb.b0);
       // all of the lane's record indices in flight at once, then its records copied straight into
       // shared memory by asynchronous 16-byte copies (no registers held), then the block masks
@@ -597,6 +605,13 @@ long long forward_warps(const Tiling& tl, long long n_tiles, int num_sms) {
 // ---------------------------------------------------------------------------------------------
 // K8
 // ---------------------------------------------------------------------------------------------
+// 1 / x for x in [1 - kAlphaMax, 1] (no range scaling needed; within 1 ulp).
+__device__ __forceinline__ float fast_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 constexpr int kBwdWarps = 4;
 constexpr int kGroup = 3;  // Gaussians whose gradient terms are summed together (3 x 9 <= 32 lanes)
 constexpr int kBwdPairs = 2;  // packed pixel pairs per lane (4 pixels, 128 per round)
@@ -610,8 +625,10 @@ struct BwdWarp {
   float acc[kChunk][9];                    // per Gaussian of the chunk: running gradient sums
 };
 
-template <int TW, int TH>
-__global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
+// SPLIT: the two warps of a pair share each item, one taking the even rounds of 128 pixels and one the
+// odd ones; the sums of both are added in that order, so the result is the same bits.
+template <int TW, int TH, bool LOAD, bool SPLIT>
+__global__ void __launch_bounds__(kBwdWarps * 32, 4) k_blend_backward(
     const ViewDev* __restrict__ views, int n_views, long long n_tiles, const uint2* __restrict__ ranges,
     const unsigned* __restrict__ vals, const ProjBuffers pb, Control* __restrict__ ctl,
     const float* __restrict__ image, const float* __restrict__ dimage, const float4* __restrict__ ckpt,
@@ -629,7 +646,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
   // moments of all the step's views); it reaches alpha through the soft count, the sum of the
   // blended Gaussians' alphas.  load_a = lambda_load / (N std), load_mu = mean; off without G_p.
   float load_a = 0.f, load_mu = 0.f;
-  if (gp != nullptr && sp->lambda_load > 0.f && ctl->gp_pixels > 0ull) {
+  if (LOAD && ctl->gp_pixels > 0ull) {
     const double np = (double)ctl->gp_pixels, mean = (double)ctl->blended / np;
     const double var = (double)ctl->gp_sq / np - mean * mean;
     if (var > 0.0) {
@@ -637,14 +654,25 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
       load_mu = (float)mean;
     }
   }
-  const bool load = load_a != 0.f;
+  // row sums of the conic's terms (2-4) carry the factors -1/2, -1, -1/2 of their products
+  const int row_gi = lane / 9, row_term = lane - 9 * row_gi;
+  const float row_scale = row_term == 3 ? -1.f : (row_term == 2 || row_term == 4 ? -0.5f : 1.f);
   const unsigned long long M = ctl->m_total;
   const long long n_ids = (long long)(M >> 5) + n_tiles + 1;
   const unsigned lt = (1u << lane) - 1u;
+  const int part = SPLIT ? warp & 1 : 0;
+  const auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp >> 1)) : "memory"); };
+  __shared__ unsigned s_claim[kBwdWarps / 2];
   for (;;) {
     long long id = 0;
-    if (lane == 0) id = (long long)atomicAdd(&ctl->bwd_work, 1u);
-    id = __shfl_sync(0xffffffffu, id, 0);
+    if (SPLIT) {
+      if (part == 0 && lane == 0) s_claim[warp >> 1] = atomicAdd(&ctl->bwd_work, 1u);
+      pair_sync();  // (also: the even warp is through with the odd one's sums)
+      id = (long long)s_claim[warp >> 1];
+    } else {
+      if (lane == 0) id = (long long)atomicAdd(&ctl->bwd_work, 1u);
+      id = __shfl_sync(0xffffffffu, id, 0);
+    }
     if (id >= n_ids) break;
     const int tp1 = chunk_tile[id];
     if (tp1 == 0) continue;
@@ -657,9 +685,9 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
     const int cnt = min(kChunk, L - base);
     const int v = view_of_tile(views, n_views, t);
     const ViewDev& V = views[v];
-    const long long local = t - V.tile_base;
-    const int tx = (int)(local % V.gx), ty = (int)(local / V.gx);
-    const long long cid = chunk_base(start, t) + k;
+    const int local = (int)(t - V.tile_base);  // (32-bit: a 64-bit division is a subroutine)
+    const int tx = local % V.gx, ty = local / V.gx;
+    const long long cid = id;
 
     unsigned long long e = 0;
     if (lane < cnt) {
@@ -690,7 +718,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
     const long long HW = (long long)V.W * V.H;
     const float* img = image + 3 * V.pix_base;
     const float* dimg = dimage + 3 * V.pix_base;
-    for (int r0 = 0; r0 < n_act; r0 += 64 * kBwdPairs) {
+    for (int r0 = part * 64 * kBwdPairs; r0 < n_act; r0 += (SPLIT ? 2 : 1) * 64 * kBwdPairs) {
       // this lane's pixels act[r0 + 32 h + lane], h = 0 .. 2 kBwdPairs - 1, pair p holding pixels
       // 2p (.x) and 2p + 1 (.y): dL/dC, the rendered colour, the state at the chunk start, minus
       // the pixel coordinates
@@ -732,7 +760,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
             }
             q[10] = -(float)px;
             q[11] = -(float)py;
-            if (load) q[12] = load_a * ((float)gp[V.pix_base + pix] - load_mu);
+            if (LOAD) q[12] = load_a * ((float)gp[V.pix_base + pix] - load_mu);
           }
         }
         d0[pp] = make_float2(st[0][0], st[1][0]);
@@ -798,9 +826,9 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
               // dL/dalpha = sum_ch dL/dC_ch (c_ch T - behind_ch / (1 - alpha)); no gradient to the
               // opacity and footprint where alpha was clamped
               const float2 cd = __ffma2_rn(cx, d0[pp], __ffma2_rn(cy, d1[pp], __fmul2_rn(cz, d2[pp])));
-              const float2 ninv = make_float2(-__fdividef(1.f, 1.f - alpha.x), -__fdividef(1.f, 1.f - alpha.y));
+              const float2 ninv = make_float2(-fast_rcp(1.f - alpha.x), -fast_rcp(1.f - alpha.y));
               float2 dal = __ffma2_rn(DS, ninv, __fmul2_rn(T[pp], cd));
-              if (load) dal = __fadd2_rn(dal, LW[pp]);  // + dL/dG_p x d alpha / d alpha
+              if (LOAD) dal = __fadd2_rn(dal, LW[pp]);  // + dL/dG_p x d alpha / d alpha
               dal.x = oG.x > kAlphaMax ? 0.f : dal.x;
               dal.y = oG.y > kAlphaMax ? 0.f : dal.y;
               const float2 dpow = __fmul2_rn(dal, alpha);
@@ -822,37 +850,35 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
               F2[pp] = n2;
             }
           }
-          // terms 2-4 of the conic: -1/2, -1, -1/2 times the accumulated products
-          S.red[9 * gi + 0][lane] = g2[0].x + g2[0].y;
-          S.red[9 * gi + 1][lane] = g2[1].x + g2[1].y;
-          S.red[9 * gi + 2][lane] = -0.5f * (g2[2].x + g2[2].y);
-          S.red[9 * gi + 3][lane] = -(g2[3].x + g2[3].y);
-          S.red[9 * gi + 4][lane] = -0.5f * (g2[4].x + g2[4].y);
 #pragma unroll
-          for (int j = 5; j < 9; ++j) S.red[9 * gi + j][lane] = g2[j].x + g2[j].y;
+          for (int j = 0; j < 9; ++j) S.red[9 * gi + j][lane] = g2[j].x + g2[j].y;
         }
         __syncwarp();
         if (lane < 9 * ng) {
           // the term's 32 values: eight 16-byte reads, four running sums (fixed order)
           const float4* row = reinterpret_cast<const float4*>(S.red[lane]);
-          float4 s4 = row[0];
+          float2 sa = make_float2(row[0].x, row[0].y), sb = make_float2(row[0].z, row[0].w);
 #pragma unroll
           for (int k = 1; k < 8; ++k) {
             const float4 x = row[k];
-            s4.x += x.x;
-            s4.y += x.y;
-            s4.z += x.z;
-            s4.w += x.w;
+            sa = __fadd2_rn(sa, make_float2(x.x, x.y));
+            sb = __fadd2_rn(sb, make_float2(x.z, x.w));
           }
-          const float sum = (s4.x + s4.y) + (s4.z + s4.w);
-          const int gi = lane / 9;
-          const int q = gi == 0 ? qs[0] : (gi == 1 ? qs[1] : qs[2]);
-          S.acc[q][lane - 9 * gi] += sum;
+          const float sum = row_scale * ((sa.x + sa.y) + (sb.x + sb.y));
+          const int q = row_gi == 0 ? qs[0] : (row_gi == 1 ? qs[1] : qs[2]);
+          S.acc[q][row_term] += sum;
         }
         __syncwarp();
       }
     }
     __syncwarp();
+    if (SPLIT) {
+      pair_sync();
+      if (part != 0) continue;
+      const BwdWarp<kPix>& O = reinterpret_cast<BwdWarp<kPix>*>(smem_raw)[warp + 1];
+#pragma unroll
+      for (int c = 0; c < 9; ++c) S.acc[lane][c] += O.acc[lane][c];
+    }
     if (lane < cnt) {
       const float* a = S.acc[lane];
       ginst[3 * e] = make_float4(a[0], a[1], a[2], a[3]);
@@ -864,41 +890,69 @@ __global__ void __launch_bounds__(kBwdWarps * 32) k_blend_backward(
 }
 
 namespace {
-template <int TW, int TH>
+template <int TW, int TH, bool LOAD, bool SPLIT>
 int& bwd_occupancy() {
   static int occ = 0;
   return occ;
 }
 
-template <int TW, int TH>
+template <int TW, int TH, bool LOAD, bool SPLIT>
 void init_backward_instance() {
   const int smem = (int)(sizeof(BwdWarp<TW * TH>) * kBwdWarps);
-  cudaFuncSetAttribute(k_blend_backward<TW, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncSetAttribute(k_blend_backward<TW, TH, LOAD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_backward<TW, TH>, kBwdWarps * 32, smem) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_backward<TW, TH, LOAD, SPLIT>, kBwdWarps * 32, smem) !=
       cudaSuccess) {
     cudaGetLastError();
     occ = 0;
   }
-  bwd_occupancy<TW, TH>() = occ > 0 ? occ : 1;
+  bwd_occupancy<TW, TH, LOAD, SPLIT>() = occ > 0 ? occ : 1;
 }
 
-template <int TW, int TH>
+template <int TW, int TH, bool LOAD, bool SPLIT>
+void launch_backward_kernel(const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
+                            const unsigned* vals, const ProjBuffers& pb, Control* ctl, const float* image,
+                            const float* dimage, const float4* ckpt, const unsigned* cmask, const int* chunk_tile,
+                            const int* tile_chunks, float4* ginst, const unsigned* gp, const StepParams* sp,
+                            int num_sms, cudaStream_t s) {
+  launch_dep(k_blend_backward<TW, TH, LOAD, SPLIT>, dim3(num_sms * bwd_occupancy<TW, TH, LOAD, SPLIT>()),
+      dim3(kBwdWarps * 32), sizeof(BwdWarp<TW * TH>) * kBwdWarps, s, views, n_views, n_tiles, ranges, vals, pb, ctl,
+      image, dimage, ckpt, cmask, chunk_tile, tile_chunks, ginst, gp, sp);
+}
+
+// A warp works on an item for 25 - 30 us (about 40 Gaussians a round, two rounds, 0.3 us each), so with
+// fewer items than pairs of warps on the chip the kernel lasts as long as one item: two warps share it.
+// With more items they keep every warp busy anyway and the second head per item is a loss.
+template <int TW, int TH, bool LOAD>
 void launch_backward_instance(const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
                               const unsigned* vals, const ProjBuffers& pb, Control* ctl, const float* image,
                               const float* dimage, const float4* ckpt, const unsigned* cmask, const int* chunk_tile,
                               const int* tile_chunks, float4* ginst, const unsigned* gp, const StepParams* sp,
-                              int num_sms, cudaStream_t s) {
-  launch_dep(k_blend_backward<TW, TH>, dim3(num_sms * bwd_occupancy<TW, TH>()), dim3(kBwdWarps * 32),
-      sizeof(BwdWarp<TW * TH>) * kBwdWarps, s, views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt,
-      cmask, chunk_tile, tile_chunks, ginst, gp, sp);
+                              long long m_cap, int num_sms, cudaStream_t s) {
+  if constexpr (TW * TH > 64 * kBwdPairs) {
+    const long long items = (m_cap >> 5) + n_tiles + 1;  // at most
+    if (items <= (long long)num_sms * bwd_occupancy<TW, TH, LOAD, true>() * (kBwdWarps / 2)) {
+      launch_backward_kernel<TW, TH, LOAD, true>(views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt,
+                                                 cmask, chunk_tile, tile_chunks, ginst, gp, sp, num_sms, s);
+      return;
+    }
+  }
+  launch_backward_kernel<TW, TH, LOAD, false>(views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt,
+                                              cmask, chunk_tile, tile_chunks, ginst, gp, sp, num_sms, s);
+}
+
+template <int TW, int TH, bool LOAD>
+void init_backward_instances() {
+  init_backward_instance<TW, TH, LOAD, false>();
+  if constexpr (TW * TH > 64 * kBwdPairs) init_backward_instance<TW, TH, LOAD, true>();
 }
 }  // namespace
 
 void init_blend_attributes() {
 #define GS_INIT(W, H, B)              \
   init_forward_instance<W, H, B>();   \
-  init_backward_instance<W, H>();
+  init_backward_instances<W, H, false>(); \
+  init_backward_instances<W, H, true>();
   GS_TILINGS(GS_INIT)
 #undef GS_INIT
 }
@@ -906,13 +960,14 @@ void init_blend_attributes() {
 void launch_blend_backward(const Tiling& tl, const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
                            const unsigned* vals, const ProjBuffers& pb, Control* ctl, const float* image,
                            const float* dimage, const float4* ckpt, const unsigned* cmask, const int* chunk_tile,
-                           const int* tile_chunks, float4* ginst, const unsigned* gp, const StepParams* sp,
-                           int num_sms, cudaStream_t s) {
+                           const int* tile_chunks, float4* ginst, const unsigned* gp, bool load, const StepParams* sp,
+                           long long m_cap, int num_sms, cudaStream_t s) {
   // the backward depends on the tile shape only
 #define GS_BWD(W, H, B)                                                                                          \
   if (tl.tw == W && tl.th == H) {                                                                               \
-    launch_backward_instance<W, H>(views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt, cmask, \
-                                   chunk_tile, tile_chunks, ginst, gp, sp, num_sms, s);                        \
+    (load ? launch_backward_instance<W, H, true> : launch_backward_instance<W, H, false>)(                     \
+        views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt, cmask, chunk_tile, tile_chunks,    \
+        ginst, gp, sp, m_cap, num_sms, s);                                                                     \
     return;                                                                                                    \
   }
   GS_TILINGS(GS_BWD)

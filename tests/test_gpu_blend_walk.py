@@ -78,3 +78,34 @@ def test_walk_edges(n, opacity, size):
     if clear.all():
         assert out["pairs"] == int(neval.sum())
     ras.close()
+
+
+@pytest.mark.parametrize("load", [0.0, 0.4])
+@pytest.mark.parametrize("tile", [(16, 16, 256), (32, 8, 256), (16, 8, 256)])
+def test_backward_item_sharing(tile, load):
+    """With few (tile, chunk) items two warps share one; with many each has its own.  Both give the same
+    bits: the first 40 Gaussians alone and the same 40 followed by enough others, too transparent to be
+    blended, that the item count passes the line."""
+    import torch
+    import paper_2503_13086_gb300 as gs
+    n, many = 40, 131_072
+    small = _scene(n, 0.5, 7)
+    big = np.zeros((59, many), np.float32)
+    big[:, :n] = small[:, :n]
+    big[:, n:] = small[:, :1]
+    big[2, n:] = 5.0  # behind them, so that the first chunks hold the same entries
+    big[10, n:] = -20.0  # opacity 2e-9: below 1/255 everywhere
+    cam = gi.identity_camera(48, 33, 16.0)
+    tgt = torch.tensor(gi.uniform_target(48, 33, 5).reshape(-1), device="cuda")
+    got = []
+    for p, k in ((small, n), (big, many)):
+        ras = gs.Raster()
+        ras.set_tiling(*tile)
+        P = torch.tensor(p, device="cuda")
+        out = ras.forward(P, k, [cam])
+        _, d = ras.loss(out["image"], tgt, 0.2, lambda_load=load)
+        got.append((out["image"].cpu().numpy(), ras.backward(P, out["image"], out["last"], d)[0].cpu().numpy()[:, :n]))
+        ras.close()
+    assert np.array_equal(got[0][0], got[1][0])
+    assert np.array_equal(got[0][1], got[1][1])
+    assert np.abs(got[0][1]).max() > 0
