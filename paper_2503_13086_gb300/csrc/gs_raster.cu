@@ -262,7 +262,7 @@ gs_status Raster::ensure_records(int stride_) {
   const long long scan_tiles = (recs + kScanTile - 1) / kScanTile;
   if ((s = zeroA.reserve(kCtlBytes + scan_tiles * 8, &bytes_in_use))) return s;
   zeroA_bytes = kCtlBytes + scan_tiles * 8;
-  if ((s = partials.reserve(n_pix * 10 * 4, &bytes_in_use)) || (s = block_sums.reserve(n_loss_blocks * 16, &bytes_in_use)))
+  if ((s = partials.reserve(n_pix * 10 * 4, &bytes_in_use)) || (s = block_sums.reserve(n_loss_blocks * 16 * (n_loss_blocks <= loss_split_blocks(num_sms) ? 3 : 1), &bytes_in_use)))
     return s;
   return GS_OK;
 }
@@ -393,7 +393,7 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
 void Raster::enqueue_loss(cudaStream_t s, const float* image, float* dimage, bool after_forward) {
   launch_loss(vd(), n_views, n_loss_blocks, image, sp(), static_cast<float*>(partials.p),
               static_cast<double*>(block_sums.p), ctl(), ledger(), dimage, after_forward ? tile_done() : nullptr,
-              forward_warps(tiling, n_tiles, num_sms), s);
+              forward_warps(tiling, n_tiles, num_sms), num_sms, s);
   mark(s, 7);
 }
 
