@@ -63,6 +63,7 @@ constexpr int kMaxViews = 32;
 // kernel launches of one optimisation step besides the sort passes: K1, K2, K3 x 2, K5 x 2, K6,
 // K7 x 2, K8, K9a x 2, K9
 constexpr int kStepLaunchesBase = 13;
+constexpr int kStepLaunchesSmall = 11;  // K3 x 2 (with K4 and K5 inside) instead of K3 x 2, K4, K5 x 2
 constexpr int kNumKernels = 9;
 constexpr int kNumEvents = kNumKernels + 1;
 constexpr size_t kCtlBytes = 1024;                                   // Control, padded
@@ -141,6 +142,9 @@ struct Raster {
   Ledger* ledger() const { return static_cast<Ledger*>(ledger_d.p); }
   void reset_ledger(cudaStream_t s) { cudaMemsetAsync(ledger_d.p, 0, sizeof(Ledger), s); }
   void read_ledger(cudaStream_t s) { cudaMemcpyAsync(ledger_h, ledger_d.p, sizeof(Ledger), cudaMemcpyDeviceToHost, s); }
+  int step_launches() const {
+    return (bin_small_cluster((long long)m_cap, tile_bits) ? kStepLaunchesSmall : kStepLaunchesBase + passes) + (dstat ? 1 : 0);
+  }
   gs_status collect_times();
   gs_status check_control();
 };

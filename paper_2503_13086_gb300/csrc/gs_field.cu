@@ -873,7 +873,7 @@ struct Field {
     last_pairs = ok ? Lg.pairs / ok : 0;
     last_blended = ok ? Lg.blended / ok : 0;
     last_instances = ok ? Lg.instances / ok : 0;
-    last_kernels = kStepLaunchesBase + R.passes + (R.dstat ? 1 : 0);
+    last_kernels = R.step_launches();
     sum_pairs += Lg.pairs;
     if (ok && Lg.last_gp_pixels) {  // Eq. 9: std of G_p over the pixels some Gaussian reaches
       const double mean = (double)Lg.last_gp_sum / (double)Lg.last_gp_pixels;

@@ -64,6 +64,13 @@ void launch_sort_pass(unsigned long long* keys0, unsigned* vals0, unsigned long 
 void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits, long long m_cap, const Control* ctl,
                    cudaStream_t s);
 
+// Small steps: owner fill, then emission, sort, ranges and tile order in one launch of a cluster of
+// `cluster` CTAs (bin_small_cluster(m_cap, tile_bits), 0: the step is not small).
+int bin_small_cluster(long long m_cap, int tile_bits);
+void launch_bin_small(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items, unsigned* inst_rec,
+                      long long n_tiles, unsigned* vals_out, uint2* ranges, int* order, int tile_bits, int cluster,
+                      const Control* ctl, cudaStream_t s);
+
 void launch_tile_order(const uint2* ranges, long long n_tiles, int* order, const Control* ctl, cudaStream_t s);
 void launch_blend_forward(const Tiling& tl, const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
                           const unsigned* vals, const ProjBuffers& pb, const StepParams* sp, Control* ctl,

@@ -371,17 +371,25 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
   unsigned long long* k1 = static_cast<unsigned long long*>(keys1.p);
   unsigned* v0 = static_cast<unsigned*>(vals0.p);
   unsigned* v1 = static_cast<unsigned*>(vals1.p);
-  launch_emit(proj(), vd(), stride, n_items, k0, v0, k1, v1, static_cast<unsigned*>(inst_rec.p),
-              hist(), tile_bits, (long long)m_cap, num_sms, ctl(), s);
-  mark(s, 3);
-  const unsigned long long sort_tiles = (m_cap + kSortTile - 1) / kSortTile;
-  for (int p = 0; p < passes; ++p)  // passes the step does not need return at once; the list ends in buffer 0
-    launch_sort_pass(k0, v0, k1, v1, hist(), sort_state() + (size_t)p * sort_tiles * kSortBins, p, tile_bits,
-                     (long long)m_cap, ctl(), s);
-  mark(s, 4);
-  launch_ranges(k0, ranges(), tile_bits, (long long)m_cap, ctl(), s);
-  launch_tile_order(ranges(), n_tiles, static_cast<int*>(order.p), ctl(), s);
-  mark(s, 5);
+  if (const int cluster = bin_small_cluster((long long)m_cap, tile_bits)) {
+    launch_bin_small(proj(), vd(), stride, n_items, static_cast<unsigned*>(inst_rec.p), n_tiles, v0, ranges(),
+                     static_cast<int*>(order.p), tile_bits, cluster, ctl(), s);
+    mark(s, 3);  // (timed as emission)
+    mark(s, 4);
+    mark(s, 5);
+  } else {
+    launch_emit(proj(), vd(), stride, n_items, k0, v0, k1, v1, static_cast<unsigned*>(inst_rec.p),
+                hist(), tile_bits, (long long)m_cap, num_sms, ctl(), s);
+    mark(s, 3);
+    const unsigned long long sort_tiles = (m_cap + kSortTile - 1) / kSortTile;
+    for (int p = 0; p < passes; ++p)  // passes the step does not need return at once; the list ends in buffer 0
+      launch_sort_pass(k0, v0, k1, v1, hist(), sort_state() + (size_t)p * sort_tiles * kSortBins, p, tile_bits,
+                       (long long)m_cap, ctl(), s);
+    mark(s, 4);
+    launch_ranges(k0, ranges(), tile_bits, (long long)m_cap, ctl(), s);
+    launch_tile_order(ranges(), n_tiles, static_cast<int*>(order.p), ctl(), s);
+    mark(s, 5);
+  }
   launch_blend_forward(tiling, vd(), n_views, n_tiles, ranges(), v0, proj(), sp(), ctl(),
                        static_cast<const int*>(order.p), image, T, last, gp, static_cast<float4*>(ckpt.p),
                        static_cast<unsigned*>(cmask.p), chunk_tile(), static_cast<int*>(tile_chunks.p),

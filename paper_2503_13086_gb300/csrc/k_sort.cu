@@ -10,6 +10,8 @@
 // host to know how many instances were emitted, so the whole chain can be graph-captured.
 // The inter-CTA waits (decoupled look-back) spin at most kSpinLimit times, then flag
 // kErrTimeout and carry on rather than hang.
+#include <atomic>
+
 #include "gs_device.cuh"
 #include "gs_engine.h"
 
@@ -444,8 +446,11 @@ __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsi
   }
 }
 
+static void init_small_attributes();
+
 void init_sort_attributes() {
   cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+  init_small_attributes();
 }
 
 void launch_sort_pass(unsigned long long* keys0, unsigned* vals0, unsigned long long* keys1, unsigned* vals1,
@@ -481,6 +486,304 @@ void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits,
   if (blocks > 4096) blocks = 4096;
   if (blocks < 1) blocks = 1;
   launch_dep(k_ranges, dim3((unsigned)blocks), dim3(256), 0, s, keys, ranges, tile_bits, ctl);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Small steps: K3's emission, K4, K5 and the tile order in one launch by one thread-block cluster.
+// Up to tens of thousands of instances the separate kernels last as long as their launches and
+// chains (5 - 8 us each for emission, every sort pass, ranges and order), whatever the bytes.  Here
+// the keys never leave the cluster: CTA r holds positions [r per, (r + 1) per) in shared memory,
+// emits them there, and each stable 8-bit pass ranks them in registers (warp by warp, as k_sort_pass),
+// exchanges the CTAs' digit totals and scatters straight into the owners' shared memory (distributed
+// shared memory).  The cluster's barriers are the hardware's; nothing spins.
+// K3 - K5 together, event times: 45 -> 28 us at 2.4k instances, 53 -> 30 at 5.2k, 60 -> 38 at 13k, 64 -> 45
+// at 29k.  The scatter's remote 8-byte stores bound it from there (records travelling beside the keys
+// took 45 instead of 30 us at 5.2k): with eight keys per thread, 69k instances, it took 79 us against 71,
+// so four keys per thread and sixteen CTAs, 65,536 instances, is where it ends.
+// ---------------------------------------------------------------------------------------------
+namespace {
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallItems = 4;                                // keys per thread at most
+constexpr int kSmallTile = kSmallThreads * kSmallItems;       // keys per CTA at most
+constexpr int kSmallMaxCluster = 16;
+constexpr int kSmallIndexBits = 16;                           // an instance's emission index, under its key
+constexpr int kSmallMaxTileBits = 14;                         // the order is one CTA's loop over the tiles
+static_assert(kSmallMaxTileBits + 32 + kSmallIndexBits <= 64, "tile, depth (at most 32 bits) and index fit a word");
+static_assert(kSmallMaxCluster * kSmallTile <= (1 << kSmallIndexBits), "the index holds every instance");
+
+struct SmallSmem {
+  unsigned long long keys[kSmallTile];
+  unsigned short cnt[kSmallWarps][kSortBins];
+  unsigned total[kSortBins];
+  unsigned gbase[kSortBins];
+  unsigned warp_sum[kSortBins / 32];
+  unsigned bucket[32], base[32];
+};
+
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// Shared-memory address of CTA `rank`'s copy of p.
+__device__ __forceinline__ unsigned cluster_addr(const void* p, unsigned rank) {
+  unsigned a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ unsigned cluster_ld_u32(unsigned a) {
+  unsigned v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long cluster_ld_u64(unsigned a) {
+  unsigned long long v;
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_st_u64(unsigned a, unsigned long long v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+}  // namespace
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_bin_small(const ProjBuffers pb, const ViewDev* __restrict__ views,
+                                                                int stride, const unsigned* __restrict__ inst_rec,
+                                                                long long n_tiles, unsigned* __restrict__ vals_out,
+                                                                uint2* __restrict__ ranges, int* __restrict__ order,
+                                                                int tile_bits, const Control* __restrict__ ctl) {
+  dep_wait();
+  dep_release();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmallSmem& S = *reinterpret_cast<SmallSmem*>(smem_raw);
+  if (ctl->overflow) return;  // every CTA of the cluster alike
+  const unsigned M = (unsigned)ctl->m_total;
+  const KeyLayout kl = key_layout(ctl, tile_bits);
+  const unsigned r = cluster_rank(), C = cluster_size();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned lt = lanemask_lt();
+  // positions per CTA: 1024 << ls, the fewest keys per thread that hold all M (M <= C kSmallTile)
+  int ls = 0;
+  while (((unsigned)kSmallThreads << ls) * C < M) ++ls;
+  const int items = 1 << ls;
+  const int per_shift = 10 + ls;
+  const unsigned per_mask = (1u << per_shift) - 1u;
+  const unsigned first = r << per_shift;          // this CTA's first position
+  const int wfirst = warp * items * 32 + lane;    // this thread's first slot: slots wfirst + 32 k
+
+  // (tile, depth) key above the instance's index: one 8-byte word per instance moves in each pass, and
+  // the record follows from the index at the end
+  unsigned long long key[kSmallItems];
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    key[k] = 0ull;
+    const unsigned e = first + (unsigned)(wfirst + 32 * k);
+    if (k < items && e < M) {
+      const unsigned rec = inst_rec[e];
+      const unsigned q = e - pb.offsets[rec];
+      const uint2 rc = pb.rect[rec];
+      const unsigned db = __float_as_uint(pb.depth[rec]);
+      const ViewDev& V = views[rec / (unsigned)stride];
+      const unsigned x0 = rc.x & 0xffffu, x1 = rc.x >> 16, y0 = rc.y & 0xffffu;
+      const unsigned w = x1 - x0;
+      const unsigned ty = y0 + q / w, tx = x0 + q % w;
+      const unsigned long long tile = (unsigned long long)(V.tile_base + (long long)ty * V.gx + tx);
+      key[k] = (((tile << kl.D) | (unsigned long long)(db - kl.dmin)) << kSmallIndexBits) | e;
+    }
+  }
+
+  for (int pass = 0; pass < kl.passes; ++pass) {
+    const int shift = kSmallIndexBits + pass * kSortBits;
+    for (int k = tid; k < kSmallWarps * kSortBins / 2; k += kSmallThreads) reinterpret_cast<unsigned*>(S.cnt)[k] = 0u;
+    __syncthreads();
+    // rank within the warp's slots, in slot order (stable)
+    unsigned rank[kSmallItems];
+#pragma unroll
+    for (int k = 0; k < kSmallItems; ++k) {
+      rank[k] = 0u;
+      if (k < items) {
+        const bool valid = first + (unsigned)(wfirst + 32 * k) < M;
+        const unsigned d = (unsigned)(key[k] >> shift) & (kSortBins - 1);
+        const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : (kSortBins + d));
+        const unsigned pre = valid ? S.cnt[warp][d] : 0u;
+        __syncwarp();
+        if (valid && (peers & lt) == 0u) S.cnt[warp][d] = (unsigned short)(pre + __popc(peers));
+        __syncwarp();
+        rank[k] = pre + __popc(peers & lt);
+      }
+    }
+    __syncthreads();
+    // per digit: exclusive prefix over the warps, and the CTA's total for the cluster
+    if (tid < kSortBins) {
+      unsigned c[kSmallWarps];
+#pragma unroll
+      for (int w = 0; w < kSmallWarps; ++w) c[w] = S.cnt[w][tid];
+      unsigned run = 0u;
+#pragma unroll
+      for (int w = 0; w < kSmallWarps; ++w) {
+        S.cnt[w][tid] = (unsigned short)run;
+        run += c[w];
+      }
+      S.total[tid] = run;
+    }
+    cluster_barrier();  // totals published; every CTA's keys of this pass are in registers
+    unsigned before = 0u, all = 0u, incl = 0u;
+    if (tid < kSortBins) {
+      for (unsigned q = 0; q < C; ++q) {
+        const unsigned t = cluster_ld_u32(cluster_addr(&S.total[tid], q));
+        before += q < r ? t : 0u;
+        all += t;
+      }
+      incl = all;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) S.warp_sum[warp] = incl;
+    }
+    __syncthreads();
+    if (tid < kSortBins) {
+      unsigned lower = 0u;
+      for (int w = 0; w < warp; ++w) lower += S.warp_sum[w];
+      S.gbase[tid] = lower + incl - all + before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSmallItems; ++k) {
+      if (k < items && first + (unsigned)(wfirst + 32 * k) < M) {
+        const unsigned d = (unsigned)(key[k] >> shift) & (kSortBins - 1);
+        const unsigned pos = S.gbase[d] + S.cnt[warp][d] + rank[k];  // < M
+        const unsigned owner = pos >> per_shift, at = pos & per_mask;
+        cluster_st_u64(cluster_addr(&S.keys[at], owner), key[k]);
+      }
+    }
+    cluster_barrier();  // every key of this CTA's positions has arrived
+#pragma unroll
+    for (int k = 0; k < kSmallItems; ++k)
+      if (k < items && first + (unsigned)(wfirst + 32 * k) < M) key[k] = S.keys[wfirst + 32 * k];
+  }
+
+  // the sorted list, and where each tile's run of it starts and ends
+#pragma unroll
+  for (int k = 0; k < kSmallItems; ++k) {
+    const int at = wfirst + 32 * k;
+    const unsigned pos = first + (unsigned)at;
+    if (k < items && pos < M) {
+      vals_out[pos] = inst_rec[(unsigned)key[k] & ((1u << kSmallIndexBits) - 1u)];
+      const int tile_shift = kSmallIndexBits + kl.D;
+      const unsigned tile = (unsigned)(key[k] >> tile_shift);
+      // neighbours: in this CTA's keys, else the last of the CTA before or the first of the CTA after
+      // (passes >= 1 put the keys into shared memory; with none there is one tile)
+      bool starts = pos == 0u, ends = pos == M - 1u;
+      if (kl.passes > 0) {
+        if (!starts) {
+          const unsigned long long p =
+              at > 0 ? S.keys[at - 1] : cluster_ld_u64(cluster_addr(&S.keys[per_mask], r - 1u));
+          starts = (unsigned)(p >> tile_shift) != tile;
+        }
+        if (!ends) {
+          const unsigned long long p =
+              (unsigned)at < per_mask ? S.keys[at + 1] : cluster_ld_u64(cluster_addr(&S.keys[0], r + 1u));
+          ends = (unsigned)(p >> tile_shift) != tile;
+        }
+      }
+      if (starts) ranges[tile].x = pos;
+      if (ends) ranges[tile].y = pos + 1u;
+    }
+  }
+  __threadfence();
+  cluster_barrier();  // the ranges are written, and no CTA reads another's shared memory any more
+  if (r != 0u) return;
+  // K6's tile order (k_tile_order): buckets by floor(log2(list length)), longest first; the ranges come
+  // from the other CTAs' SMs, so they are read through L2
+  if (tid < 32) S.bucket[tid] = 0u;
+  __syncthreads();
+  const auto bucket_of = [&](long long t) {
+    const unsigned long long rg = ld_relaxed_u64(reinterpret_cast<const unsigned long long*>(ranges + t));
+    const unsigned L = (unsigned)(rg >> 32) - (unsigned)rg;
+    return min(L ? 32 - __clz(L) : 0, 31);
+  };
+  for (long long t = tid; t < n_tiles; t += kSmallThreads) atomicAdd(&S.bucket[bucket_of(t)], 1u);
+  __syncthreads();
+  if (tid == 0) {
+    unsigned run = 0u;
+    for (int b = 31; b >= 0; --b) {
+      S.base[b] = run;
+      run += S.bucket[b];
+    }
+  }
+  __syncthreads();
+  for (long long t = tid; t < n_tiles; t += kSmallThreads) order[atomicAdd(&S.base[bucket_of(t)], 1u)] = (int)t;
+}
+
+// Cluster size for up to m_cap instances, 0 when the step is not small.  Set at start-up: a size the device
+// cannot place (16 is beyond the portable 8) is not used.
+static std::atomic<int> g_small_max_cluster{0};
+
+int bin_small_cluster(long long m_cap, int tile_bits) {
+  const int most = g_small_max_cluster;
+  if (tile_bits > kSmallMaxTileBits || m_cap > (long long)most * kSmallTile) return 0;
+  int c = 1;
+  while (c < most && (long long)c * kSmallThreads < m_cap) c <<= 1;  // as few keys per thread as the cluster allows
+  return c;
+}
+
+namespace {
+cudaLaunchConfig_t small_config(int cluster, cudaLaunchAttribute* attr, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cluster);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.dynamicSmemBytes = sizeof(SmallSmem);
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cfg;
+}
+}  // namespace
+
+static void init_small_attributes() {
+  cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem));
+  cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  int best = 0;
+  for (int c = 1; c <= kSmallMaxCluster; c <<= 1) {
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = small_config(c, attr, nullptr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_bin_small, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      break;
+    }
+    if (n < 1) break;
+    best = c;
+  }
+  g_small_max_cluster = best;
+}
+
+void launch_bin_small(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items, unsigned* inst_rec,
+                      long long n_tiles, unsigned* vals_out, uint2* ranges, int* order, int tile_bits, int cluster,
+                      const Control* ctl, cudaStream_t s) {
+  if (n_items <= 0) return;
+  launch_dep(k_fill_owner, dim3((unsigned)((n_items + 255) / 256)), dim3(256), 0, s, pb.count, pb.offsets, n_items,
+      inst_rec, ctl);
+  cudaLaunchAttribute attr[2];
+  const cudaLaunchConfig_t cfg = small_config(cluster, attr, s);
+  cudaLaunchKernelEx(&cfg, k_bin_small, pb, views, stride, (const unsigned*)inst_rec, n_tiles, vals_out, ranges, order,
+                     tile_bits, ctl);
 }
 
 // ---------------------------------------------------------------------------------------------
