@@ -243,6 +243,7 @@ class Raster:
         _check(self._lib.gs_raster_create(ctypes.byref(h)))
         self._h = h
         self._sizes = None
+        self._n = 0  # Gaussians of the last forward
         self.generation = 0  # bumped by every forward (the workspace keeps only the latest one)
 
     def close(self):
@@ -272,6 +273,7 @@ class Raster:
                                            _cams(cams), len(cams), bgv, _ptr(image), _ptr(T), _ptr(last), _ptr(gp),
                                            ctypes.byref(pairs)))
         self._sizes = sizes
+        self._n = int(n)
         self.generation += 1
         return dict(image=image, T=T, last=last, gp=gp, pairs=int(pairs.value), sizes=sizes)
 
@@ -287,7 +289,9 @@ class Raster:
 
     def backward(self, params, image, last, dimage, want_grad2d=False, stream=None):
         torch = _torch()
-        grads = torch.zeros_like(params)
+        grads = torch.empty_like(params)  # the call writes every Gaussian's 59 rows; the padding is zero
+        if self._n < params.shape[1]:
+            grads[:, self._n:].zero_()
         grad2d = None
         if want_grad2d:
             grad2d = torch.zeros(len(self._sizes) * params.shape[1] * 9, device=params.device, dtype=torch.float32)
