@@ -174,15 +174,22 @@ __device__ __forceinline__ bool geo_forward(const ViewDev& V, const float mu[3],
 }
 
 // ---------------------------------------------------------------------------------------------
-// K1: projection forward.  grid = (ceil(stride / 256), views); one thread per (view, Gaussian).
+// K1: projection forward; one thread per (view, Gaussian), a view's CTA next to the other views' CTAs over
+// the same 128 Gaussians, so that the parameter rows come from DRAM once and then from L2 (with all
+// Gaussians of a view before the next view: 251 -> 193 us for nine views of 500k).  Bound by the latency of
+// its two rounds of loads (geometry, then SH): 64 registers hold a channel's 16 SH coefficients in flight
+// per thread, and eight 128-thread CTAs per SM still keep more bytes in flight than DRAM needs; at 40
+// registers with an L2 prefetch loop over the rows instead, the loads went out a few at a time: 193 -> 172 us
+// for the nine views, 257 -> 189 for three of 1.5M, 19.6 -> 17.0 at 200k, 13.5 -> 8.2 at 20k.  (64-thread CTAs:
+// 183 us; one thread looping over the views: 330 us, the loop's loads are hoisted and spill.)
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 6) k_project(const float* __restrict__ params, int stride,
+__global__ void __launch_bounds__(128, 8) k_project(const float* __restrict__ params, int stride,
                                                  const StepParams* __restrict__ sp,
-                                                 const ViewDev* __restrict__ views, ProjBuffers out) {
+                                                 const ViewDev* __restrict__ views, int n_views, ProjBuffers out) {
   dep_wait();
   dep_release();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int v = blockIdx.y;
+  const int v = (int)(blockIdx.x % (unsigned)n_views);
+  const int i = (int)(blockIdx.x / (unsigned)n_views * blockDim.x + threadIdx.x);
   if (i >= stride) return;
   const long long rec = (long long)v * stride + i;
   const int n = sp->n;
@@ -234,29 +241,23 @@ __global__ void __launch_bounds__(256, 6) k_project(const float* __restrict__ pa
   d0 *= dl;
   d1 *= dl;
   d2 *= dl;
-  // the 48 SH coefficient rows and the opacity logit on their way to L2 at once (no register held):
-  // the loads below, which the compiler issues a few at a time (40 registers keep six CTAs per SM,
-  // so a 200k-Gaussian view is one wave), then find them there instead of making one DRAM round
-  // trip per batch
-  {
-    const float* pf = params + 10ll * stride + i;
-#pragma unroll 1
-    for (int k = 0; k < 49; ++k, pf += stride) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
-  }
+  const float logit = __ldg(params + 10 * stride + i);
   float Y[16];
   sh_basis(d0, d1, d2, Y);
   float col[3];
   unsigned clampbits = 0u;
 #pragma unroll
   for (int ch = 0; ch < 3; ++ch) {
-    float acc = 0.f;
+    float acc = 0.f, c[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) acc += Y[k] * __ldg(params + (11 + 3 * k + ch) * stride + i);
+    for (int k = 0; k < 16; ++k) c[k] = __ldg(params + (11 + 3 * k + ch) * stride + i);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) acc += Y[k] * c[k];
     acc += 0.5f;
     if (acc < 0.f) clampbits |= 1u << ch;
     col[ch] = fmaxf(acc, 0.f);
   }
-  const float opac = 1.f / (1.f + __expf(-__ldg(params + 10 * stride + i)));
+  const float opac = 1.f / (1.f + __expf(-logit));
   // alpha = opacity * exp(power) reaches 1/255 only where power >= thr = -ln(255 opacity), i.e.
   // inside the ellipse d^T conic d <= 2 ln(255 opacity); its axis-aligned half extents are
   // sqrt(2 ln(255 opacity) cov_xx), sqrt(.. cov_yy).  Widened by 0.1 % + 0.01 px so no pixel the
@@ -966,8 +967,8 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ params, const 
 
 void launch_project(const float* params, int stride, int n_views, const StepParams* sp, const ViewDev* views,
                     const ProjBuffers& out, cudaStream_t s) {
-  dim3 grid((stride + 255) / 256, n_views);
-  launch_dep(k_project, dim3(grid), dim3(256), 0, s, params, stride, sp, views, out);
+  const dim3 grid((unsigned)((stride + 127) / 128) * (unsigned)n_views);
+  launch_dep(k_project, grid, dim3(128), 0, s, params, stride, sp, views, n_views, out);
 }
 
 void launch_project_backward(float* params, int stride, int n_views, const StepParams* sp, const ViewDev* views,
