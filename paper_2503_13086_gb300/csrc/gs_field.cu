@@ -1481,14 +1481,21 @@ gs_status gs_render(gs_field* ff, const gs_camera* cam, float* out_rgb, float* o
   P.n_views = 1;
   for (int a = 0; a < 3; ++a) P.bg[a] = f->cfg.bg[a];
   P.adam = 0;
-  R.reset_ledger(f->stream);
-  R.upload(f->stream);
-  if ((s = R.enqueue_forward_head(f->stream, static_cast<float*>(f->params.p), f->stride, true))) return s;
-  if ((s = R.enqueue_forward_tail(f->stream, out_rgb, out_T, static_cast<unsigned*>(f->step_last.p), nullptr, false))) return s;
-  f->sized_for_views = false;
-  R.enqueue_readback(f->stream);
-  cudaError_t e = cudaStreamSynchronize(f->stream);
-  if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));
+  // as gs_raster_forward: no round trip for the instance count while the buffers hold it
+  bool sized = !R.sized_before;
+  for (;;) {
+    R.reset_ledger(f->stream);
+    R.upload(f->stream);
+    if ((s = R.enqueue_forward_head(f->stream, static_cast<float*>(f->params.p), f->stride, sized))) return s;
+    if ((s = R.ensure_instances(R.m_cap))) return s;
+    if ((s = R.enqueue_forward_tail(f->stream, out_rgb, out_T, static_cast<unsigned*>(f->step_last.p), nullptr, false))) return s;
+    f->sized_for_views = false;
+    R.enqueue_readback(f->stream);
+    cudaError_t e = cudaStreamSynchronize(f->stream);
+    if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("render: ") + cudaGetErrorString(e));
+    if (sized || !R.ctl_h->overflow) break;
+    sized = true;
+  }
   return R.check_control();
 }
 

@@ -357,6 +357,7 @@ gs_status Raster::enqueue_forward_head(cudaStream_t s, const float* params, int 
       gs_status st = ensure_instances(m + m / 4 + 1024);
       if (st) return st;
     }
+    sized_before = true;
   }
   return GS_OK;
 }
@@ -506,22 +507,29 @@ gs_status gs_raster_forward(gs_raster* rr, void* stream, const float* params, in
   P.n_views = n_views;
   for (int k = 0; k < 3; ++k) P.bg[k] = bg ? bg[k] : 0.f;
   P.adam = 0;
-  r->reset_ledger(s);
-  r->upload(s);
-  if ((st = r->enqueue_forward_head(s, params, (int)stride, true))) return st;
-  if ((st = r->ensure_instances(r->m_cap))) return st;
-  if ((st = r->enqueue_forward_tail(s, out_image, out_T, out_last, out_gp, false))) return st;
-  r->have_forward = true;
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("forward launch: ") + cudaGetErrorString(e));
-  if (out_pairs) {
+  // With instance buffers from an earlier forward and a result the host waits for anyway, the whole chain is
+  // enqueued at once and the instance count is looked at with that result: the round trip between the
+  // scan and the emission leaves the device idle for about 20 us.  If the count did not fit, the scan
+  // made every later kernel return, and the forward runs again with the count read in between.
+  bool sized = out_pairs == nullptr || !r->sized_before;
+  for (;;) {
+    r->reset_ledger(s);
+    r->upload(s);
+    if ((st = r->enqueue_forward_head(s, params, (int)stride, sized))) return st;
+    if ((st = r->ensure_instances(r->m_cap))) return st;
+    if ((st = r->enqueue_forward_tail(s, out_image, out_T, out_last, out_gp, false))) return st;
+    r->have_forward = true;
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("forward launch: ") + cudaGetErrorString(e));
+    if (!out_pairs) return GS_OK;
     r->enqueue_readback(s);
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("forward: ") + cudaGetErrorString(e));
-    *out_pairs = r->ctl_h->pairs;
-    if ((st = r->check_control())) return st;
+    if (sized || !r->ctl_h->overflow) break;
+    sized = true;
   }
-  return GS_OK;
+  *out_pairs = r->ctl_h->pairs;
+  return r->check_control();
 }
 
 gs_status gs_raster_loss(gs_raster* rr, void* stream, const float* image, const float* target,
