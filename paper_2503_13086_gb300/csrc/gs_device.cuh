@@ -83,6 +83,8 @@ struct Control {
   unsigned int fwd_work;
   unsigned int loss_done;
   unsigned int fwd_done;        // blend-forward warps past their last counter update
+  unsigned int listed;          // records with instances (large steps list them)
+  unsigned int list_ticket;
   unsigned int order_count[32];  // tiles per list-length bucket (long-first schedule)
   double loss_view[32];         // per-view loss of the last step
   double loss;                  // batch loss (mean over views)

@@ -92,6 +92,7 @@ struct Raster {
   bool zeroB_pending = true;  // zeroB still to be cleared by the forward tail
   DevBuf xyo, conic, rgb, depth, radius, rect, count, offsets, clamp, g2s;
   DevBuf keys0, keys1, vals0, vals1, ginst, ckpt, cmask, order, tile_chunks;
+  DevBuf list0, list1, place_of;  // large steps: listed records (two buffers), where each one's instances go
   DevBuf inst_rec, carry;  // instance -> record, K9a partials
   DevBuf partials, block_sums;
   DevBuf ledger_d;  // Ledger of the current run of steps
@@ -120,6 +121,19 @@ struct Raster {
   uint2* ranges() const;
   int* chunk_tile() const;
   unsigned* tile_done() const;  // per tile: 1 once the blend forward finished it
+  unsigned long long* list_state(int k) const;  // look-back states of the list (0) and of its count scan (1)
+  // Large steps sort depth and tile apart (k_sort.cu).  Against the (tile, depth) passes, K2 - K4 together:
+  // 529 -> 380 us at 6.5M instances of 2.0M listed records, 218 -> 201 at 2.8M of 0.86M, 159 -> 154 at 1.6M of
+  // 0.5M, but 121 -> 130 at 1.2M and 114 -> 129 at 1.0M on a 160 x 100 image (one pass fewer without it), where
+  // the two more launches and the list cost more than the passes they shorten.
+  static constexpr long long kLargeRecords = 1ll << 19, kLargeInstances = 3ll << 20;  // least records, capacity
+  bool large() const {
+    const long long n_rec = (long long)n_views * stride;
+    return n_rec >= kLargeRecords && n_rec < (1ll << 31) && tile_bits <= 8 * (kMaxSortPasses - kDepthPasses) &&
+           (long long)m_cap >= kLargeInstances;
+  }
+  bool list_ready = false;  // ensure_records made the list's buffers for the current views
+  bool list_built = false;  // the last forward head listed its records (not one whose m_cap grew after ensure_records)
   ProjBuffers proj() const;
   const StepParams* sp() const { return static_cast<const StepParams*>(sp_d.p); }
   const ViewDev* vd() const { return static_cast<const ViewDev*>(views_d.p); }
@@ -144,7 +158,10 @@ struct Raster {
   void reset_ledger(cudaStream_t s) { cudaMemsetAsync(ledger_d.p, 0, sizeof(Ledger), s); }
   void read_ledger(cudaStream_t s) { cudaMemcpyAsync(ledger_h, ledger_d.p, sizeof(Ledger), cudaMemcpyDeviceToHost, s); }
   int step_launches() const {
-    return (bin_small_cluster((long long)m_cap, tile_bits) ? kStepLaunchesSmall : kStepLaunchesBase + passes) + (dstat ? 1 : 0);
+    int k = kStepLaunchesBase + passes;
+    if (bin_small_cluster((long long)m_cap, tile_bits)) k = kStepLaunchesSmall;
+    else if (list_built) k = kStepLaunchesBase + 2 + kDepthPasses + word_tile_passes(tile_bits);
+    return k + (dstat ? 1 : 0);
   }
   gs_status collect_times();
   gs_status check_control();

@@ -32,6 +32,8 @@ constexpr int kSortTile = kSortThreads * kSortItems;  // keys per onesweep CTA
 constexpr int kSortBits = 8;
 constexpr int kSortBins = 1 << kSortBits;
 constexpr int kMaxSortPasses = 8;
+constexpr int kDepthPasses = 4;    // large steps: passes over the listed records' 32 depth bits
+constexpr int kWordMinBlocks = 2;  // resident word-sort CTAs per SM the registers must allow
 
 // Tile shape of the binning and blending, and the number of sorted Gaussians K6 stages in shared
 // memory per round.  Only the shapes/batches in tiling_candidates() are compiled.
@@ -54,15 +56,24 @@ void launch_adam(float* params, const float* grads, float* m, float* v, int n, i
                  cudaStream_t s);
 
 void launch_scan(const unsigned* in, unsigned* out, long long n_items, unsigned long long* state, Control* ctl,
-                 unsigned long long m_cap, Ledger* ledger, cudaStream_t s, const float* depth = nullptr);
+                 unsigned long long m_cap, Ledger* ledger, cudaStream_t s, const float* depth = nullptr,
+                 unsigned long long* list = nullptr, unsigned long long* list_state = nullptr);
 void launch_emit(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items, unsigned long long* keys0,
                  unsigned* vals0, unsigned long long* keys1, unsigned* vals1, unsigned* inst_rec, unsigned* hist,
                  int tile_bits, long long m_cap, int num_sms, const Control* ctl, cudaStream_t s);
 void launch_sort_pass(unsigned long long* keys0, unsigned* vals0, unsigned long long* keys1, unsigned* vals1,
                       const unsigned* hist, unsigned* state, int pass, int tile_bits, long long m_cap, Control* ctl,
                       cudaStream_t s);
-void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits, long long m_cap, const Control* ctl,
-                   cudaStream_t s);
+// shift: bit where the tile starts in a key, 0: the step's key layout
+void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits, int shift, long long m_cap,
+                   const Control* ctl, cudaStream_t s);
+// Large steps: depth sort of the listed records (launch_scan's list), emission in that order, tile sort.
+int word_tile_passes(int tile_bits);
+void launch_sort_large(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items,
+                       unsigned long long* list0, unsigned long long* list1, unsigned* place_of,
+                       unsigned long long* list_state, unsigned long long* words0, unsigned long long* words1,
+                       unsigned* vals_out, unsigned* inst_rec, unsigned* hist, unsigned* state, int tile_bits,
+                       long long m_cap, int num_sms, Control* ctl, cudaStream_t s);
 
 // Small steps: owner fill, then emission, sort, ranges and tile order in one launch of a cluster of
 // `cluster` CTAs (bin_small_cluster(m_cap, tile_bits), 0: the step is not small).

@@ -162,7 +162,7 @@ Raster::Raster() {
 
 Raster::~Raster() {
   DevBuf* all[] = {&sp_d, &views_d, &ledger_d, &zeroA, &zeroB, &xyo, &conic, &rgb, &depth, &radius, &rect, &count, &offsets,
-                   &clamp, &g2s, &keys0, &keys1, &vals0, &vals1, &ginst, &inst_rec, &carry, &ckpt, &cmask, &order, &tile_chunks, &partials, &block_sums, &own_image,
+                   &clamp, &g2s, &keys0, &keys1, &vals0, &vals1, &ginst, &inst_rec, &carry, &list0, &list1, &place_of, &ckpt, &cmask, &order, &tile_chunks, &partials, &block_sums, &own_image,
                    &own_last, &own_dimage};
   for (DevBuf* b : all) b->release(&bytes_in_use);
   if (sp_h) cudaFreeHost(sp_h);
@@ -176,6 +176,10 @@ Raster::~Raster() {
 Control* Raster::ctl() const { return reinterpret_cast<Control*>(zeroA.p); }
 unsigned long long* Raster::scan_state() const {
   return reinterpret_cast<unsigned long long*>(static_cast<char*>(zeroA.p) + kCtlBytes);
+}
+unsigned long long* Raster::list_state(int k) const {
+  const long long tiles = ((long long)n_views * stride + kScanTile - 1) / kScanTile;
+  return scan_state() + (size_t)(1 + k) * tiles;
 }
 unsigned* Raster::hist() const { return reinterpret_cast<unsigned*>(zeroB.p); }
 unsigned* Raster::sort_state() const {
@@ -260,8 +264,15 @@ gs_status Raster::ensure_records(int stride_) {
       (s = clamp.reserve(recs, &bytes_in_use)) || (s = g2s.reserve(recs * 36, &bytes_in_use)))
     return s;
   const long long scan_tiles = (recs + kScanTile - 1) / kScanTile;
-  if ((s = zeroA.reserve(kCtlBytes + scan_tiles * 8, &bytes_in_use))) return s;
-  zeroA_bytes = kCtlBytes + scan_tiles * 8;
+  stride = stride_;
+  list_ready = false;
+  const long long states = large() ? 3 : 1;
+  if ((s = zeroA.reserve(kCtlBytes + states * scan_tiles * 8, &bytes_in_use))) return s;
+  zeroA_bytes = kCtlBytes + states * scan_tiles * 8;
+  if (large() && ((s = list0.reserve(recs * 8, &bytes_in_use)) || (s = list1.reserve(recs * 8, &bytes_in_use)) ||
+                  (s = place_of.reserve(recs * 4, &bytes_in_use))))
+    return s;
+  list_ready = large();
   if ((s = partials.reserve(n_pix * 10 * 4, &bytes_in_use)) || (s = block_sums.reserve(n_loss_blocks * 16 * (n_loss_blocks <= loss_split_blocks(num_sms) ? 3 : 1), &bytes_in_use)))
     return s;
   return GS_OK;
@@ -296,6 +307,12 @@ gs_status Raster::ensure_instances(unsigned long long m) {
     return s;
   const unsigned long long sort_tiles = (m_cap + kSortTile - 1) / kSortTile;
   sort_state_bytes = (size_t)passes * sort_tiles * kSortBins * 4;
+  if (large()) {
+    const unsigned long long rec_tiles = ((unsigned long long)n_views * stride + kSortTile - 1) / kSortTile;
+    sort_state_bytes = std::max<size_t>(
+        sort_state_bytes,
+        ((size_t)kDepthPasses * rec_tiles + (size_t)word_tile_passes(tile_bits) * sort_tiles) * kSortBins * 4);
+  }
   ranges_bytes = (size_t)n_tiles * 8;
   chunk_bytes = (size_t)n_ids * 4;
   zeroB_bytes = kHistBytes + sort_state_bytes + ranges_bytes + chunk_bytes + (size_t)n_tiles * 4;
@@ -345,8 +362,10 @@ gs_status Raster::enqueue_forward_head(cudaStream_t s, const float* params, int 
   launch_project(params, stride_, n_views, sp(), vd(), proj(), s);
   mark(s, 1);
   const long long n_items = (long long)n_views * stride_;
+  list_built = list_ready;
   launch_scan(proj().count, proj().offsets, n_items, scan_state(), ctl(), size_exactly ? ~0ull : m_cap, ledger(), s,
-              proj().depth);
+              proj().depth, list_built ? static_cast<unsigned long long*>(list0.p) : nullptr,
+              list_built ? list_state(0) : nullptr);
   mark(s, 2);
   if (size_exactly) {
     cudaMemcpyAsync(ctl_h, ctl(), sizeof(Control), cudaMemcpyDeviceToHost, s);
@@ -378,6 +397,16 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
     mark(s, 3);  // (timed as emission)
     mark(s, 4);
     mark(s, 5);
+  } else if (list_built) {
+    launch_sort_large(proj(), vd(), stride, n_items, static_cast<unsigned long long*>(list0.p),
+                      static_cast<unsigned long long*>(list1.p), static_cast<unsigned*>(place_of.p), list_state(1), k0, k1,
+                      v0, static_cast<unsigned*>(inst_rec.p), hist(), sort_state(), tile_bits, (long long)m_cap, num_sms,
+                      ctl(), s);
+    mark(s, 3);  // (emission and sorts timed together, as the sort)
+    mark(s, 4);
+    launch_ranges(k0, ranges(), tile_bits, 32, (long long)m_cap, ctl(), s);
+    launch_tile_order(ranges(), n_tiles, static_cast<int*>(order.p), ctl(), s);
+    mark(s, 5);
   } else {
     launch_emit(proj(), vd(), stride, n_items, k0, v0, k1, v1, static_cast<unsigned*>(inst_rec.p),
                 hist(), tile_bits, (long long)m_cap, num_sms, ctl(), s);
@@ -387,7 +416,7 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
       launch_sort_pass(k0, v0, k1, v1, hist(), sort_state() + (size_t)p * sort_tiles * kSortBins, p, tile_bits,
                        (long long)m_cap, ctl(), s);
     mark(s, 4);
-    launch_ranges(k0, ranges(), tile_bits, (long long)m_cap, ctl(), s);
+    launch_ranges(k0, ranges(), tile_bits, 0, (long long)m_cap, ctl(), s);
     launch_tile_order(ranges(), n_tiles, static_cast<int*>(order.p), ctl(), s);
     mark(s, 5);
   }

@@ -36,41 +36,115 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 // K2: single-pass exclusive scan with decoupled look-back.  Tiles are taken in launch order via
 // an atomic ticket, so every tile a CTA waits on belongs to a CTA that is already running.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned* __restrict__ in, unsigned* __restrict__ out,
+// SCAN_COMPACT also lists the records with instances, (depth bits << 32 | record) in record order, for the
+// depth presort of large steps: a second warp runs the same look-back for the number of listed records.
+// SCAN_LIST scans the counts of the listed records in list order (n_items = the list's length, device-
+// resident) and writes each record's offset to out[record].
+enum ScanMode { SCAN_PLAIN, SCAN_COMPACT, SCAN_LIST };
+
+// Decoupled look-back by a whole warp: lane l reads the status of tile j - l, so one round trip covers up
+// to 32 predecessors.  Publishes the tile's total, returns the sum before it.
+__device__ __forceinline__ unsigned long long scan_lookback(unsigned long long* __restrict__ state, unsigned tile,
+                                                            unsigned long long total, int lane,
+                                                            Control* __restrict__ ctl, unsigned spin_limit) {
+  unsigned long long excl = 0;
+  if (tile == 0) {
+    if (lane == 0) st_relaxed_u64(&state[0], kScanPrefix | total);
+    return 0ull;
+  }
+  if (lane == 0) st_relaxed_u64(&state[tile], kScanAgg | total);
+  long long j = (long long)tile - 1;
+  unsigned spins = 0;
+  for (;;) {
+    const long long idx = j - lane;
+    const unsigned long long sv = idx >= 0 ? ld_relaxed_u64(&state[idx]) : kScanPrefix;
+    const unsigned long long flag = sv & ~kScanValMask;
+    const unsigned notready = __ballot_sync(0xffffffffu, flag == 0ull);
+    const unsigned isprefix = __ballot_sync(0xffffffffu, flag == kScanPrefix);
+    const unsigned stop = notready | isprefix;
+    const int first = stop ? __ffs(stop) - 1 : 32;  // lanes below it hold aggregates
+    const bool take = lane < first || (lane == first && ((isprefix >> lane) & 1u));
+    unsigned long long v = take ? (sv & kScanValMask) : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    excl += v;
+    if (first < 32 && ((isprefix >> first) & 1u)) break;
+    j -= first;
+    if (first < 32 && ++spins > spin_limit) {
+      if (lane == 0) atomicOr(&ctl->error, kErrTimeout);
+      break;
+    }
+  }
+  if (lane == 0) st_relaxed_u64(&state[tile], kScanPrefix | (excl + total));
+  return excl;
+}
+
+// The large steps' scan of all records takes tiles of 8192: the look-back advances 32 tiles per round trip, so
+// with 2048 the chain over 4.5M records set the time (49 against 40 us).  The scan of the listed ones keeps
+// 2048: its gather wants the CTAs (10 us slower with 8192 at 0.9M).
+constexpr int kLargeScanThreads = 512, kLargeScanItems = 16;
+constexpr int kLargeScanTile = kLargeScanThreads * kLargeScanItems;
+
+template <int MODE>
+__global__ void __launch_bounds__(MODE == SCAN_COMPACT ? kLargeScanThreads : kScanThreads) k_scan(const unsigned* __restrict__ in, unsigned* __restrict__ out,
                                                        long long n_items, unsigned long long* __restrict__ state,
                                                        Control* __restrict__ ctl, unsigned long long m_cap,
                                                        Ledger* __restrict__ ledger, const float* __restrict__ depth,
-                                                       unsigned spin_limit) {
+                                                       unsigned spin_limit, unsigned long long* __restrict__ list,
+                                                       unsigned long long* __restrict__ list_state) {
+  constexpr int kThr = MODE == SCAN_COMPACT ? kLargeScanThreads : kScanThreads;
+  constexpr int kItems = MODE == SCAN_COMPACT ? kLargeScanItems : kScanItems;
+  constexpr int kTileItems = kThr * kItems;
   dep_wait();
   dep_release();
   __shared__ unsigned s_tile;
-  __shared__ unsigned s_warp[kScanThreads / 32];
+  __shared__ unsigned s_warp[kThr / 32], s_lwarp[kThr / 32];
   __shared__ unsigned long long s_excl;
-  if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->scan_ticket, 1u);
+  __shared__ unsigned s_lexcl;
+  if (MODE == SCAN_LIST) {
+    if (ctl->overflow) return;
+    n_items = (long long)ctl->listed;
+  }
+  if (threadIdx.x == 0) s_tile = atomicAdd(MODE == SCAN_LIST ? &ctl->list_ticket : &ctl->scan_ticket, 1u);
   __syncthreads();
   const unsigned tile = s_tile;
-  const long long num_tiles = (n_items + kScanTile - 1) / kScanTile;
-  const long long base = (long long)tile * kScanTile + (long long)threadIdx.x * kScanItems;
-  unsigned x[kScanItems];
-  if (base + kScanItems <= n_items) {
-    const uint4 a = *reinterpret_cast<const uint4*>(in + base);
-    const uint4 b = *reinterpret_cast<const uint4*>(in + base + 4);
-    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+  const long long num_tiles = (n_items + kTileItems - 1) / kTileItems;
+  if (MODE == SCAN_LIST && (long long)tile >= num_tiles) return;
+  const long long base = (long long)tile * kTileItems + (long long)threadIdx.x * kItems;
+  unsigned x[kItems], rec[kItems];
+  if (MODE == SCAN_LIST) {
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) rec[k] = base + k < n_items ? (unsigned)list[base + k] : 0u;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) x[k] = base + k < n_items ? in[rec[k]] : 0u;
+  } else if (base + kItems <= n_items) {
+#pragma unroll
+    for (int k = 0; k < kItems; k += 4) {
+      const uint4 a = *reinterpret_cast<const uint4*>(in + base + k);
+      x[k] = a.x;
+      x[k + 1] = a.y;
+      x[k + 2] = a.z;
+      x[k + 3] = a.w;
+    }
   } else {
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) x[k] = (base + k < n_items) ? in[base + k] : 0u;
+    for (int k = 0; k < kItems; ++k) x[k] = (base + k < n_items) ? in[base + k] : 0u;
   }
-  unsigned tsum = 0;
+  unsigned tsum = 0, tlist = 0;
 #pragma unroll
-  for (int k = 0; k < kScanItems; ++k) tsum += x[k];
+  for (int k = 0; k < kItems; ++k) {
+    tsum += x[k];
+    tlist += x[k] != 0u;
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (depth) {  // range of the depth bits of the records with instances (the sort key layout)
+  unsigned db[kItems];
+  if (MODE != SCAN_LIST && depth) {  // range of the depth bits of the records with instances (the sort key layout)
     unsigned dmax = 0u, dnot = 0u;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k)
+    for (int k = 0; k < kItems; ++k)
       if (x[k]) {
         const unsigned b = __float_as_uint(depth[base + k]);
+        if (MODE == SCAN_COMPACT) db[k] = b;
         dmax = max(dmax, b);
         dnot = max(dnot, ~b);
       }
@@ -82,58 +156,36 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned* __restric
     }
   }
   // block-wide exclusive scan of the per-thread sums
-  unsigned incl = tsum;
+  unsigned incl = tsum, lincl = tlist;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const unsigned y = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += y;
+    const unsigned z = MODE == SCAN_COMPACT ? __shfl_up_sync(0xffffffffu, lincl, d) : 0u;
+    if (lane >= d) {
+      incl += y;
+      lincl += z;
+    }
   }
-  if (lane == 31) s_warp[warp] = incl;
+  if (lane == 31) {
+    s_warp[warp] = incl;
+    if (MODE == SCAN_COMPACT) s_lwarp[warp] = lincl;
+  }
   __syncthreads();
-  if (warp == 0) {
-    unsigned w = lane < kScanThreads / 32 ? s_warp[lane] : 0u;
+  if (warp == 0 || (MODE == SCAN_COMPACT && warp == 1)) {
+    unsigned* sums = warp == 0 ? s_warp : s_lwarp;
+    const unsigned w = lane < kThr / 32 ? sums[lane] : 0u;
     unsigned wi = w;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const unsigned y = __shfl_up_sync(0xffffffffu, wi, d);
       if (lane >= d) wi += y;
     }
-    if (lane < kScanThreads / 32) s_warp[lane] = wi - w;  // exclusive warp offsets
-    const unsigned total = __shfl_sync(0xffffffffu, wi, kScanThreads / 32 - 1);
-    // decoupled look-back by the whole warp: lane l reads the status of tile j - l, so one round
-    // trip covers up to 32 predecessors
-    unsigned long long excl = 0;
-    if (tile == 0) {
-      if (lane == 0) st_relaxed_u64(&state[0], kScanPrefix | (unsigned long long)total);
-    } else {
-      if (lane == 0) st_relaxed_u64(&state[tile], kScanAgg | (unsigned long long)total);
-      long long j = (long long)tile - 1;
-      unsigned spins = 0;
-      for (;;) {
-        const long long idx = j - lane;
-        const unsigned long long sv = idx >= 0 ? ld_relaxed_u64(&state[idx]) : kScanPrefix;
-        const unsigned long long flag = sv & ~kScanValMask;
-        const unsigned notready = __ballot_sync(0xffffffffu, flag == 0ull);
-        const unsigned isprefix = __ballot_sync(0xffffffffu, flag == kScanPrefix);
-        const unsigned stop = notready | isprefix;
-        const int first = stop ? __ffs(stop) - 1 : 32;  // lanes below it hold aggregates
-        const bool take = lane < first || (lane == first && ((isprefix >> lane) & 1u));
-        unsigned long long v = take ? (sv & kScanValMask) : 0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        excl += v;
-        if (first < 32 && ((isprefix >> first) & 1u)) break;
-        j -= first;
-        if (first < 32 && ++spins > spin_limit) {
-          if (lane == 0) atomicOr(&ctl->error, kErrTimeout);
-          break;
-        }
-      }
-      if (lane == 0) st_relaxed_u64(&state[tile], kScanPrefix | (excl + total));
-    }
-    if (lane == 0) {
+    if (lane < kThr / 32) sums[lane] = wi - w;  // exclusive warp offsets
+    const unsigned total = __shfl_sync(0xffffffffu, wi, kThr / 32 - 1);
+    const unsigned long long excl = scan_lookback(warp == 0 ? state : list_state, tile, total, lane, ctl, spin_limit);
+    if (lane == 0 && warp == 0) {
       s_excl = excl;
-      if ((long long)tile == num_tiles - 1) {
+      if (MODE != SCAN_LIST && (long long)tile == num_tiles - 1) {
         const unsigned long long m = excl + total;
         ctl->m_total = m;
         // an overflow skips this step; an earlier skipped step of the run skips it too
@@ -147,21 +199,39 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned* __restric
         }
       }
     }
+    if (MODE == SCAN_COMPACT && lane == 0 && warp == 1) {
+      s_lexcl = (unsigned)excl;
+      if ((long long)tile == num_tiles - 1) ctl->listed = (unsigned)excl + total;
+    }
   }
   __syncthreads();
   unsigned run = (unsigned)s_excl + s_warp[warp] + (incl - tsum);
-  if (base + kScanItems <= n_items) {
-    unsigned y[kScanItems];
+  if (MODE == SCAN_COMPACT) {
+    unsigned pos = s_lexcl + s_lwarp[warp] + (lincl - tlist);
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-      y[k] = run;
+    for (int k = 0; k < kItems; ++k)
+      if (x[k]) list[pos++] = ((unsigned long long)db[k] << 32) | (unsigned)(base + k);
+  }
+  if (MODE == SCAN_LIST) {
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+      if (base + k < n_items) out[rec[k]] = run;
       run += x[k];
     }
-    *reinterpret_cast<uint4*>(out + base) = make_uint4(y[0], y[1], y[2], y[3]);
-    *reinterpret_cast<uint4*>(out + base + 4) = make_uint4(y[4], y[5], y[6], y[7]);
+  } else if (base + kItems <= n_items) {
+#pragma unroll
+    for (int k = 0; k < kItems; k += 4) {
+      uint4 y;
+      y.x = run;
+      y.y = y.x + x[k];
+      y.z = y.y + x[k + 1];
+      y.w = y.z + x[k + 2];
+      run = y.w + x[k + 3];
+      *reinterpret_cast<uint4*>(out + base + k) = y;
+    }
   } else {
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
+    for (int k = 0; k < kItems; ++k) {
       if (base + k < n_items) out[base + k] = run;
       run += x[k];
     }
@@ -169,10 +239,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const unsigned* __restric
 }
 
 void launch_scan(const unsigned* in, unsigned* out, long long n_items, unsigned long long* state, Control* ctl,
-                 unsigned long long m_cap, Ledger* ledger, cudaStream_t s, const float* depth) {
-  const long long tiles = (n_items + kScanTile - 1) / kScanTile;
-  launch_dep(k_scan, dim3((unsigned)tiles), dim3(kScanThreads), 0, s, in, out, n_items, state, ctl, m_cap, ledger,
-      depth, kSpinLimit);
+                 unsigned long long m_cap, Ledger* ledger, cudaStream_t s, const float* depth,
+                 unsigned long long* list, unsigned long long* list_state) {
+  const int tile = list ? kLargeScanTile : kScanTile;
+  launch_dep(list ? k_scan<SCAN_COMPACT> : k_scan<SCAN_PLAIN>, dim3((unsigned)((n_items + tile - 1) / tile)),
+      dim3(list ? kLargeScanThreads : kScanThreads), 0, s, in, out, n_items, state, ctl, m_cap, ledger, depth, kSpinLimit,
+      list, list_state);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -282,10 +354,55 @@ struct SortSmem {
   unsigned long long keys[kSortTile];
   unsigned vals[kSortTile];
   unsigned cnt[kSortThreads / 32][kSortBins];
+  unsigned mask[kSortThreads / 32][kSortBins];
   unsigned bstart[kSortBins];
   unsigned gbase[kSortBins];
   unsigned tile;
 };
+
+// Decoupled look-back of one digit: publishes the tile's total and returns the sum over the tiles before.
+__device__ __forceinline__ unsigned sort_lookback(unsigned* __restrict__ state, unsigned tile, int d, unsigned total,
+                                                  Control* __restrict__ ctl, unsigned spin_limit) {
+  unsigned excl = 0u;
+      unsigned* st = state + (unsigned long long)tile * kSortBins + d;
+      if (tile == 0) {
+        st_relaxed_u32(st, kSortPrefix | total);
+      } else {
+        st_relaxed_u32(st, kSortAgg | total);
+        // look-back over windows of kLookBack predecessors (their loads in flight together)
+        constexpr int kLookBack = 8;
+        long long j = (long long)tile - 1;
+        unsigned spins = 0;
+        bool done = false;
+        while (!done) {
+          unsigned sv[kLookBack];
+  #pragma unroll
+          for (int w = 0; w < kLookBack; ++w)
+            sv[w] = j - w >= 0 ? ld_relaxed_u32(state + (unsigned long long)(j - w) * kSortBins + d) : kSortPrefix;
+          int used = 0;
+          bool wait = false;
+  #pragma unroll
+          for (int w = 0; w < kLookBack; ++w) {
+            if (done || wait) continue;
+            const unsigned flag = sv[w] & ~kSortValMask;
+            if (flag == 0u) {
+              wait = true;
+              continue;
+            }
+            excl += sv[w] & kSortValMask;
+            ++used;
+            if (flag == kSortPrefix) done = true;
+          }
+          j -= used;
+          if (wait && ++spins > spin_limit) {
+            atomicOr(&ctl->error, kErrTimeout);
+            break;
+          }
+        }
+        st_relaxed_u32(st, kSortPrefix | (excl + total));
+      }
+  return excl;
+}
 
 __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsigned long long* __restrict__ keys0,
                                                             unsigned* __restrict__ vals0,
@@ -309,7 +426,10 @@ __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsi
   unsigned* __restrict__ vout = from1 ? vals0 : vals1;
   const unsigned long long M = ctl->m_total;
   if (threadIdx.x == 0) S.tile = atomicAdd(&ctl->sort_ticket[pass], 1u);
-  for (int k = threadIdx.x; k < (kSortThreads / 32) * kSortBins; k += kSortThreads) (&S.cnt[0][0])[k] = 0u;
+  for (int k = threadIdx.x; k < (kSortThreads / 32) * kSortBins; k += kSortThreads) {
+    (&S.cnt[0][0])[k] = 0u;
+    (&S.mask[0][0])[k] = 0u;
+  }
   __syncthreads();
   const unsigned tile = S.tile;
   const unsigned long long tile0 = (unsigned long long)tile * kSortTile;
@@ -334,10 +454,15 @@ __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsi
     const unsigned long long idx = wbase + (unsigned)(r * 32 + lane);
     const bool valid = idx < M;
     const unsigned d = (unsigned)(key[r] >> shift) & (kSortBins - 1);
-    const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : (kSortBins + d));
+    if (valid) atomicOr(&S.mask[warp][d], 1u << lane);
+    __syncwarp();
+    const unsigned peers = valid ? S.mask[warp][d] : 0u;
     const unsigned pre = valid ? S.cnt[warp][d] : 0u;
     __syncwarp();
-    if (valid && (peers & lt) == 0u) S.cnt[warp][d] = pre + __popc(peers);
+    if (valid && (peers & lt) == 0u) {
+      S.cnt[warp][d] = pre + __popc(peers);
+      S.mask[warp][d] = 0u;
+    }
     __syncwarp();
     rank[r] = pre + __popc(peers & lt);
   }
@@ -358,43 +483,7 @@ __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsi
       run += c;
     }
     total = run;
-    unsigned* st = state + (unsigned long long)tile * kSortBins + d;
-    if (tile == 0) {
-      st_relaxed_u32(st, kSortPrefix | total);
-    } else {
-      st_relaxed_u32(st, kSortAgg | total);
-      // look-back over windows of kLookBack predecessors (their loads in flight together)
-      constexpr int kLookBack = 8;
-      long long j = (long long)tile - 1;
-      unsigned spins = 0;
-      bool done = false;
-      while (!done) {
-        unsigned sv[kLookBack];
-#pragma unroll
-        for (int w = 0; w < kLookBack; ++w)
-          sv[w] = j - w >= 0 ? ld_relaxed_u32(state + (unsigned long long)(j - w) * kSortBins + d) : kSortPrefix;
-        int used = 0;
-        bool wait = false;
-#pragma unroll
-        for (int w = 0; w < kLookBack; ++w) {
-          if (done || wait) continue;
-          const unsigned flag = sv[w] & ~kSortValMask;
-          if (flag == 0u) {
-            wait = true;
-            continue;
-          }
-          excl += sv[w] & kSortValMask;
-          ++used;
-          if (flag == kSortPrefix) done = true;
-        }
-        j -= used;
-        if (wait && ++spins > spin_limit) {
-          atomicOr(&ctl->error, kErrTimeout);
-          break;
-        }
-      }
-      st_relaxed_u32(st, kSortPrefix | (excl + total));
-    }
+    excl = sort_lookback(state, tile, d, total, ctl, spin_limit);
     // digit base = exclusive scan of the global histogram; CTA digit start = exclusive scan of
     // the CTA totals
     h = hist[pass * kSortBins + d];
@@ -446,12 +535,6 @@ __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsi
   }
 }
 
-static void init_small_attributes();
-
-void init_sort_attributes() {
-  cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
-  init_small_attributes();
-}
 
 void launch_sort_pass(unsigned long long* keys0, unsigned* vals0, unsigned long long* keys1, unsigned* vals1,
                       const unsigned* hist, unsigned* state, int pass, int tile_bits, long long m_cap, Control* ctl,
@@ -462,16 +545,237 @@ void launch_sort_pass(unsigned long long* keys0, unsigned* vals0, unsigned long 
 }
 
 // ---------------------------------------------------------------------------------------------
+// Large steps: depth first, then tiles.  The order of an instance within its tile depends on its record
+// alone (depth, then index), and there are two to four instances per listed record.  So the listed
+// records are sorted by depth (four 8-bit passes over 8-byte words), their counts scanned in that order,
+// the instances emitted to the places that scan gives them, and only the tile digits (one to three
+// passes) then run over the instances, on 8-byte words (tile << 32 | record) instead of a 12-byte key and
+// value through five or six passes.  The list is the same: both sorts are stable and the records start
+// in index order.  The word's own slots, which K9a reads, stay in record order.
+// ---------------------------------------------------------------------------------------------
+struct WordSmem {
+  unsigned long long keys[kSortTile];
+  unsigned cnt[kSortThreads / 32][kSortBins];
+  unsigned mask[kSortThreads / 32][kSortBins];
+  unsigned bstart[kSortBins];
+  unsigned gbase[kSortBins];
+  unsigned tile;
+};
+
+// One stable pass over the digit at `shift` of n 8-byte words; as k_sort_pass, without values.  vout
+// (nullable): also the words' low halves.
+__global__ void __launch_bounds__(kSortThreads, kWordMinBlocks) k_sort_pass_words(
+    const unsigned long long* __restrict__ kin, unsigned long long* __restrict__ kout, unsigned* __restrict__ vout,
+    int by_record, const unsigned* __restrict__ hist, unsigned* __restrict__ state, int shift, int ticket,
+    Control* __restrict__ ctl, unsigned spin_limit) {
+  dep_wait();
+  dep_release();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  WordSmem& S = *reinterpret_cast<WordSmem*>(smem_raw);
+  if (ctl->overflow) return;
+  const unsigned long long M = by_record ? (unsigned long long)ctl->listed : ctl->m_total;
+  if (threadIdx.x == 0) S.tile = atomicAdd(&ctl->sort_ticket[ticket], 1u);
+  for (int k = threadIdx.x; k < (kSortThreads / 32) * kSortBins; k += kSortThreads) {
+    (&S.cnt[0][0])[k] = 0u;
+    (&S.mask[0][0])[k] = 0u;
+  }
+  __syncthreads();
+  const unsigned tile = S.tile;
+  const unsigned long long tile0 = (unsigned long long)tile * kSortTile;
+  if (tile0 >= M) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = lanemask_lt();
+  unsigned long long key[kSortItems];
+  unsigned rank[kSortItems];
+  const unsigned long long wbase = tile0 + (unsigned long long)warp * (kSortItems * 32);
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r) {
+    const unsigned long long idx = wbase + (unsigned)(r * 32 + lane);
+    key[r] = idx < M ? kin[idx] : ~0ull;
+  }
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r) {
+    const bool valid = wbase + (unsigned)(r * 32 + lane) < M;
+    const unsigned d = (unsigned)(key[r] >> shift) & (kSortBins - 1);
+    if (valid) atomicOr(&S.mask[warp][d], 1u << lane);
+    __syncwarp();
+    const unsigned peers = valid ? S.mask[warp][d] : 0u;
+    const unsigned pre = valid ? S.cnt[warp][d] : 0u;
+    __syncwarp();
+    if (valid && (peers & lt) == 0u) {
+      S.cnt[warp][d] = pre + __popc(peers);
+      S.mask[warp][d] = 0u;
+    }
+    __syncwarp();
+    rank[r] = pre + __popc(peers & lt);
+  }
+  __syncthreads();
+  __shared__ unsigned s_wa[kSortBins / 32], s_wb[kSortBins / 32];
+  const int d = threadIdx.x;
+  const bool digit = d < kSortBins;
+  unsigned total = 0u, excl = 0u, h = 0u, a = 0u, b = 0u;
+  if (digit) {
+    unsigned run = 0;
+#pragma unroll
+    for (int w = 0; w < kSortThreads / 32; ++w) {
+      const unsigned c = S.cnt[w][d];
+      S.cnt[w][d] = run;
+      run += c;
+    }
+    total = run;
+    h = hist[d];
+    excl = sort_lookback(state, tile, d, total, ctl, spin_limit);
+    a = h;
+    b = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned ya = __shfl_up_sync(0xffffffffu, a, o);
+      const unsigned yb = __shfl_up_sync(0xffffffffu, b, o);
+      if (lane >= o) {
+        a += ya;
+        b += yb;
+      }
+    }
+    if (lane == 31) {
+      s_wa[warp] = a;
+      s_wb[warp] = b;
+    }
+  }
+  __syncthreads();
+  if (digit) {
+    unsigned pa = 0, pb = 0;
+    for (int w = 0; w < warp; ++w) {
+      pa += s_wa[w];
+      pb += s_wb[w];
+    }
+    S.gbase[d] = pa + a - h + excl;
+    S.bstart[d] = pb + b - total;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kSortItems; ++r) {
+    if (wbase + (unsigned)(r * 32 + lane) < M) {
+      const unsigned dd = (unsigned)(key[r] >> shift) & (kSortBins - 1);
+      S.keys[S.bstart[dd] + S.cnt[warp][dd] + rank[r]] = key[r];
+    }
+  }
+  __syncthreads();
+  const unsigned tile_count = (unsigned)min((unsigned long long)kSortTile, M - tile0);
+  for (unsigned k = threadIdx.x; k < tile_count; k += kSortThreads) {
+    const unsigned long long kk = S.keys[k];
+    const unsigned dd = (unsigned)(kk >> shift) & (kSortBins - 1);
+    const unsigned gpos = S.gbase[dd] + (k - S.bstart[dd]);
+    kout[gpos] = kk;
+    if (vout) vout[gpos] = (unsigned)kk;
+  }
+}
+
+// The four digit histograms of the listed records' depths.
+__global__ void __launch_bounds__(1024) k_depth_hist(const unsigned long long* __restrict__ list,
+                                                     unsigned* __restrict__ hist, const Control* __restrict__ ctl) {
+  dep_wait();
+  dep_release();
+  __shared__ unsigned s_hist[kDepthPasses][kSortBins];
+  if (ctl->overflow) return;
+  for (int k = threadIdx.x; k < kDepthPasses * kSortBins; k += blockDim.x) (&s_hist[0][0])[k] = 0u;
+  __syncthreads();
+  const unsigned n = ctl->listed;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned db = (unsigned)(list[i] >> 32);
+#pragma unroll
+    for (int p = 0; p < kDepthPasses; ++p) atomicAdd(&s_hist[p][(db >> (p * kSortBits)) & (kSortBins - 1)], 1u);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < kDepthPasses * kSortBins; k += blockDim.x) {
+    const unsigned c = (&s_hist[0][0])[k];
+    if (c) atomicAdd(hist + k, c);
+  }
+}
+
+// K3 of a large step: instance e (record order) of record r goes to place_of[r] + (its index in r).
+__global__ void __launch_bounds__(512) k_emit_words(const ProjBuffers pb, const ViewDev* __restrict__ views, int stride,
+                                                    const unsigned* __restrict__ place_of,
+                                                    unsigned long long* __restrict__ words,
+                                                    const unsigned* __restrict__ inst_rec, unsigned* __restrict__ hist,
+                                                    int tile_passes, const Control* __restrict__ ctl) {
+  dep_wait();
+  dep_release();
+  __shared__ unsigned s_hist[kMaxSortPasses - kDepthPasses][kSortBins];
+  if (ctl->overflow) return;
+  for (int k = threadIdx.x; k < tile_passes * kSortBins; k += blockDim.x) (&s_hist[0][0])[k] = 0u;
+  __syncthreads();
+  const unsigned long long M = ctl->m_total;
+  for (unsigned long long e = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; e < M;
+       e += (unsigned long long)gridDim.x * blockDim.x) {
+    const unsigned rec = inst_rec[e];
+    const unsigned k = (unsigned)e - pb.offsets[rec];
+    const uint2 rc = pb.rect[rec];
+    const unsigned at = place_of[rec] + k;
+    const ViewDev& V = views[rec / (unsigned)stride];
+    const unsigned x0 = rc.x & 0xffffu, x1 = rc.x >> 16, y0 = rc.y & 0xffffu;
+    const unsigned w = x1 - x0;
+    const unsigned ty = y0 + k / w, tx = x0 + k % w;
+    const unsigned tile = (unsigned)(V.tile_base + (long long)ty * V.gx + tx);
+    words[at] = ((unsigned long long)tile << 32) | rec;
+    for (int p = 0; p < tile_passes; ++p) atomicAdd(&s_hist[p][(tile >> (p * kSortBits)) & (kSortBins - 1)], 1u);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < tile_passes * kSortBins; k += blockDim.x) {
+    const unsigned c = (&s_hist[0][0])[k];
+    if (c) atomicAdd(hist + k, c);
+  }
+}
+
+static void init_small_attributes();
+
+void init_sort_attributes() {
+  cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+  cudaFuncSetAttribute(k_sort_pass_words, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem));
+  init_small_attributes();
+}
+
+int word_tile_passes(int tile_bits) { return tile_bits <= kSortBits ? 1 : (tile_bits + kSortBits - 1) / kSortBits; }
+
+void launch_sort_large(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items,
+                       unsigned long long* list0, unsigned long long* list1, unsigned* place_of,
+                       unsigned long long* list_state, unsigned long long* words0, unsigned long long* words1,
+                       unsigned* vals_out, unsigned* inst_rec, unsigned* hist, unsigned* state, int tile_bits,
+                       long long m_cap, int num_sms, Control* ctl, cudaStream_t s) {
+  const unsigned rec_tiles = (unsigned)((n_items + kSortTile - 1) / kSortTile);
+  const unsigned inst_tiles = (unsigned)((m_cap + kSortTile - 1) / kSortTile);
+  launch_dep(k_depth_hist, dim3((unsigned)(2 * num_sms)), dim3(1024), 0, s, list0, hist, ctl);
+  for (int p = 0; p < kDepthPasses; ++p)
+    launch_dep(k_sort_pass_words, dim3(rec_tiles), dim3(kSortThreads), sizeof(WordSmem), s, (p & 1) ? list1 : list0,
+        (p & 1) ? list0 : list1, nullptr, 1, hist + p * kSortBins, state + (size_t)p * rec_tiles * kSortBins,
+        32 + p * kSortBits, p, ctl, kSpinLimit);
+  launch_dep(k_scan<SCAN_LIST>, dim3((unsigned)((n_items + kScanTile - 1) / kScanTile)), dim3(kScanThreads), 0, s,
+      pb.count, place_of, 0ll, list_state, ctl, 0ull, nullptr, nullptr, kSpinLimit, list0, nullptr);
+  launch_dep(k_fill_owner, dim3((unsigned)((n_items + 255) / 256)), dim3(256), 0, s, pb.count, pb.offsets, n_items,
+      inst_rec, ctl);
+  const int tp = word_tile_passes(tile_bits);
+  // the last pass ends in words0: start in words[tp & 1]
+  launch_dep(k_emit_words, dim3((unsigned)(4 * num_sms)), dim3(512), 0, s, pb, views, stride, place_of,
+      (tp & 1) ? words1 : words0, inst_rec, hist + kDepthPasses * kSortBins, tp, ctl);
+  unsigned* tstate = state + (size_t)kDepthPasses * rec_tiles * kSortBins;
+  for (int p = 0; p < tp; ++p) {
+    const bool from1 = ((tp - p) & 1) != 0;
+    launch_dep(k_sort_pass_words, dim3(inst_tiles), dim3(kSortThreads), sizeof(WordSmem), s, from1 ? words1 : words0,
+        from1 ? words0 : words1, p == tp - 1 ? vals_out : nullptr, 0, hist + (kDepthPasses + p) * kSortBins,
+        tstate + (size_t)p * inst_tiles * kSortBins, 32 + p * kSortBits, kDepthPasses + p, ctl, kSpinLimit);
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
 // K5: per-tile [start, end) of the sorted list.  Empty tiles keep the [0, 0) the step's clear
 // left them.  Grid-stride over the device-resident instance count.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_ranges(const unsigned long long* __restrict__ keys, uint2* __restrict__ ranges,
-                                                int tile_bits, const Control* __restrict__ ctl) {
+                                                int tile_bits, int shift, const Control* __restrict__ ctl) {
   dep_wait();
   dep_release();
   if (ctl->overflow) return;
   const unsigned long long M = ctl->m_total;
-  const int D = key_layout(ctl, tile_bits).D;
+  const int D = shift ? shift : key_layout(ctl, tile_bits).D;  // where the tile starts in the key
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < M;
        i += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned tile = (unsigned)(keys[i] >> D);
@@ -480,12 +784,12 @@ __global__ void __launch_bounds__(256) k_ranges(const unsigned long long* __rest
   }
 }
 
-void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits, long long m_cap, const Control* ctl,
-                   cudaStream_t s) {
+void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits, int shift, long long m_cap,
+                   const Control* ctl, cudaStream_t s) {
   long long blocks = (m_cap + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   if (blocks < 1) blocks = 1;
-  launch_dep(k_ranges, dim3((unsigned)blocks), dim3(256), 0, s, keys, ranges, tile_bits, ctl);
+  launch_dep(k_ranges, dim3((unsigned)blocks), dim3(256), 0, s, keys, ranges, tile_bits, shift, ctl);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -829,10 +1133,10 @@ gs_status run_wait_probe(unsigned spin_limit, unsigned out_error[2], float out_m
         check(cudaMemcpyAsync(ctl_b, &cb, sizeof(Control), cudaMemcpyHostToDevice, st), "cudaMemcpyAsync") &&
         check(cudaMemcpyAsync(hist, &h0, sizeof(unsigned), cudaMemcpyHostToDevice, st), "cudaMemcpyAsync")) {
       cudaEventRecord(ev[0], st);
-      k_scan<<<1, kScanThreads, 0, st>>>(reinterpret_cast<const unsigned*>(d + off_in),
+      k_scan<SCAN_PLAIN><<<1, kScanThreads, 0, st>>>(reinterpret_cast<const unsigned*>(d + off_in),
                                          reinterpret_cast<unsigned*>(d + off_out), (long long)n_scan,
                                          reinterpret_cast<unsigned long long*>(d + off_state_a), ctl_a, ~0ull,
-                                         nullptr, nullptr, spin_limit);
+                                         nullptr, nullptr, spin_limit, nullptr, nullptr);
       cudaEventRecord(ev[1], st);
       k_sort_pass<<<1, kSortThreads, sizeof(SortSmem), st>>>(
           reinterpret_cast<unsigned long long*>(d + off_k0), reinterpret_cast<unsigned*>(d + off_v0),
