@@ -920,9 +920,10 @@ void launch_backward_kernel(const ViewDev* views, int n_views, long long n_tiles
       image, dimage, ckpt, cmask, chunk_tile, tile_chunks, ginst, gp, sp);
 }
 
-// A warp works on an item for 25 - 30 us (about 40 Gaussians a round, two rounds, 0.3 us each), so with
-// fewer items than pairs of warps on the chip the kernel lasts as long as one item: two warps share it.
-// With more items they keep every warp busy anyway and the second head per item is a loss.
+// A warp works on an item for 25 - 45 us (about 40 Gaussians in its two rounds, 0.6 - 1 us each), so with few
+// items the kernel lasts as long as the slowest of them: two warps share each up to eight items per pair
+// of warps on the chip.  One warp against two: 33 -> 25 us at 220 items (at most, by the buffers), 39 -> 26 at
+// 1.6k, 45 -> 43 at 3.6k, 60 -> 56 at 5.9k, 81 -> 80 at 9.0k; with 14k and more the second head per item shows.
 template <int TW, int TH, bool LOAD>
 void launch_backward_instance(const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
                               const unsigned* vals, const ProjBuffers& pb, Control* ctl, const float* image,
@@ -931,7 +932,7 @@ void launch_backward_instance(const ViewDev* views, int n_views, long long n_til
                               long long m_cap, int num_sms, cudaStream_t s) {
   if constexpr (TW * TH > 64 * kBwdPairs) {
     const long long items = (m_cap >> 5) + n_tiles + 1;  // at most
-    if (items <= (long long)num_sms * bwd_occupancy<TW, TH, LOAD, true>() * (kBwdWarps / 2)) {
+    if (items <= 8ll * num_sms * bwd_occupancy<TW, TH, LOAD, true>() * (kBwdWarps / 2)) {
       launch_backward_kernel<TW, TH, LOAD, true>(views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt,
                                                  cmask, chunk_tile, tile_chunks, ginst, gp, sp, num_sms, s);
       return;

@@ -88,7 +88,7 @@ def test_backward_item_sharing(tile, load):
     blended, that the item count passes the line."""
     import torch
     import paper_2503_13086_gb300 as gs
-    n, many = 40, 131_072
+    n, many = 40, 393_216
     small = _scene(n, 0.5, 7)
     big = np.zeros((59, many), np.float32)
     big[:, :n] = small[:, :n]
