@@ -801,9 +801,10 @@ void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits,
 // exchanges the CTAs' digit totals and scatters straight into the owners' shared memory (distributed
 // shared memory).  The cluster's barriers are the hardware's; nothing spins.
 // K3 - K5 together, event times: 45 -> 28 us at 2.4k instances, 53 -> 30 at 5.2k, 60 -> 38 at 13k, 64 -> 45
-// at 29k.  The scatter's remote 8-byte stores bound it from there (records travelling beside the keys
-// took 45 instead of 30 us at 5.2k): with eight keys per thread, 69k instances, it took 79 us against 71,
-// so four keys per thread and sixteen CTAs, 65,536 instances, is where it ends.
+// at 29k.  From there the work of sixteen SMs bounds it: with eight keys per thread, 69k instances, it took
+// 79 us against 71 (also with each digit's run staged so that it leaves as consecutive words; records
+// travelling beside the keys took 45 instead of 30 us at 5.2k), so four keys per thread and sixteen CTAs,
+// 65,536 instances, is where it ends.
 // ---------------------------------------------------------------------------------------------
 namespace {
 constexpr int kSmallThreads = 1024;
