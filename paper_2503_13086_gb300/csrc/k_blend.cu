@@ -12,8 +12,8 @@
 // and publishes it on an mbarrier, so staging overlaps the other warps' walk and a fast warp can run
 // a job ahead of the tile's slowest block instead of waiting for it at a CTA barrier.  Jobs are
 // walked in chunks of 32.  A warp skips a Gaussian outright when the bounding box of its 1/255 cutoff
-// ellipse misses the warp's block (warp-uniform).  The others are taken two at a time without a branch:
-// every lane evaluates both exponents and alphas, then blends them in list order under predicates.  A
+// ellipse misses the warp's block (warp-uniform).  The others are taken two at a time (four when the tiles
+// are few, see few_tiles) without a branch: every lane evaluates both exponents and alphas, then blends them in list order under predicates.  A
 // pixel's walk is one dependent chain, and the longest lists set the kernel's duration from a few
 // thousand Gaussians up, so what counts is the chain's length per candidate: with a branch per test
 // (cutoff, alpha, stop) it was about 300 cycles, in this form about 210 when a CTA has its SM to itself,
@@ -172,10 +172,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
 }
 }  // namespace
 
-template <int TW, int TH, int BATCH>
-__global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
+// DEEP: candidates of a chunk evaluated together in a round of the walk (with 2 a lone last one alone).
+template <int TW, int TH, int BATCH, int DEEP>
+__device__ __forceinline__ void blend_forward(
     const ViewDev* __restrict__ views, int n_views, long long n_tiles, const uint2* __restrict__ ranges,
-    const unsigned* __restrict__ vals, const ProjBuffers pb, const StepParams* __restrict__ sp,
+    const unsigned* __restrict__ vals, const ProjBuffers& pb, const StepParams* __restrict__ sp,
     Control* __restrict__ ctl, const int* __restrict__ order, float* __restrict__ image, float* __restrict__ Tout,
     unsigned* __restrict__ last_out, unsigned* __restrict__ gp_out, float4* __restrict__ ckpt,
     unsigned* __restrict__ cmask, int* __restrict__ chunk_tile, int* __restrict__ tile_chunks,
@@ -459,6 +460,24 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
       unsigned mask = 0u;
       // One straight line per candidate, two candidates in flight: every lane evaluates both
       // exponents and alphas, then they are blended in list order under predicates.
+      if (DEEP > 2) {
+        while (cand) {
+          unsigned bit[DEEP];
+          int q[DEEP];
+#pragma unroll
+          for (int u = 0; u < DEEP; ++u) {
+            bit[u] = cand & (0u - cand);
+            q[u] = bit[u] ? 31 - __clz(bit[u]) : q[u ? u - 1 : 0];
+            cand ^= bit[u];
+          }
+          Cand e[DEEP];
+#pragma unroll
+          for (int u = 0; u < DEEP; ++u) e[u] = eval(buf, c0 + q[u]);
+          bool stop = false;
+#pragma unroll
+          for (int u = 0; u < DEEP; ++u) stop |= blend(e[u], e[u].use && bit[u] != 0u && !stop, bit[u], jg0 + q[u], mask);
+        }
+      }
       while (cand) {
         const unsigned bit0 = cand & (0u - cand);
         const int q0 = 31 - __clz(bit0);
@@ -514,6 +533,28 @@ __global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(
   }
 }
 
+#define GS_FORWARD_PARAMS                                                                                             \
+  const ViewDev *__restrict__ views, int n_views, long long n_tiles, const uint2 *__restrict__ ranges,                \
+      const unsigned *__restrict__ vals, const ProjBuffers pb, const StepParams *__restrict__ sp,                     \
+      Control *__restrict__ ctl, const int *__restrict__ order, float *__restrict__ image, float *__restrict__ Tout,  \
+      unsigned *__restrict__ last_out, unsigned *__restrict__ gp_out, float4 *__restrict__ ckpt,                      \
+      unsigned *__restrict__ cmask, int *__restrict__ chunk_tile, int *__restrict__ tile_chunks,                      \
+      unsigned *__restrict__ tile_done
+#define GS_FORWARD_ARGS                                                                                               \
+  views, n_views, n_tiles, ranges, vals, pb, sp, ctl, order, image, Tout, last_out, gp_out, ckpt, cmask, chunk_tile, \
+      tile_chunks, tile_done
+
+template <int TW, int TH, int BATCH>
+__global__ void __launch_bounds__(TW * TH, 1024 / (TW * TH)) k_blend_forward(GS_FORWARD_PARAMS) {
+  blend_forward<TW, TH, BATCH, 2>(GS_FORWARD_ARGS);
+}
+
+constexpr int kDeep = 4;
+template <int TW, int TH, int BATCH>
+__global__ void __launch_bounds__(TW * TH, 512 / (TW * TH)) k_blend_forward_few(GS_FORWARD_PARAMS) {
+  blend_forward<TW, TH, BATCH, kDeep>(GS_FORWARD_ARGS);
+}
+
 void launch_tile_order(const uint2* ranges, long long n_tiles, int* order, const Control* ctl, cudaStream_t s) {
   if (n_tiles <= 0) return;
   launch_dep(k_tile_order, dim3(1), dim3(1024), 0, s, ranges, n_tiles, order, ctl);
@@ -521,26 +562,44 @@ void launch_tile_order(const uint2* ranges, long long n_tiles, int* order, const
 
 namespace {
 // Resident CTAs per SM of one K6 instance (persistent grid = that x SMs), set at start-up.
-template <int TW, int TH, int BATCH>
+template <int TW, int TH, int BATCH, bool FEW>
 int& fwd_occupancy() {
   static int occ = 0;
   return occ;
 }
 
-template <int TW, int TH, int BATCH>
-void init_forward_instance() {
+template <int TW, int TH, int BATCH, bool FEW>
+void init_forward_kernel() {
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_forward<TW, TH, BATCH>, TW * TH, 0) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &occ, FEW ? k_blend_forward_few<TW, TH, BATCH> : k_blend_forward<TW, TH, BATCH>, TW * TH, 0) != cudaSuccess) {
     cudaGetLastError();
     occ = 0;
   }
-  fwd_occupancy<TW, TH, BATCH>() = occ > 0 ? occ : 1;
+  fwd_occupancy<TW, TH, BATCH, FEW>() = occ > 0 ? occ : 1;
 }
+
+template <int TW, int TH, int BATCH>
+void init_forward_instance() {
+  init_forward_kernel<TW, TH, BATCH, false>();
+  init_forward_kernel<TW, TH, BATCH, true>();
+}
+
+// With few tiles the longest lists' chains are the kernel's duration and most of the chip idles, so four
+// candidates go into each round of the walk at 128 registers and two CTAs per SM (per candidate about 130
+// instead of 210 cycles).  Up to 16 tiles per SM: 616 -> 452 us on a 128 x 96 image of 150k Gaussians (48
+// tiles), 164 -> 133 at 300 x 200 of 120k (247), 110 -> 84 at 160 x 120 of 30k, 32 -> 26 at 128 x 97 of 3k, 70 -> 57 at
+// 640 x 360 of 60k (920), 91 -> 75 at 1000 x 600 of 200k (2394), 61 -> 62 at 960 x 540 of 60k (2040).  With 4346
+// tiles it depends on the lists, which the host does not know (262 against 330 us at 1.9M, but 123 against
+// 110 at 200k with large Gaussians over the image), and with 8160 and more the lost occupancy shows (148
+// against 118, 1042 against 751 on nine views).  Eight per round: 471 us on the 48 tiles.
+bool few_tiles(long long n_tiles, int num_sms) { return n_tiles <= 16ll * num_sms; }
 
 // Persistent grid of one K6 instance: every resident CTA, at most one per tile.
 template <int TW, int TH, int BATCH>
 long long forward_grid(long long n_tiles, int num_sms) {
-  long long grid = (long long)num_sms * fwd_occupancy<TW, TH, BATCH>();
+  const int occ = few_tiles(n_tiles, num_sms) ? fwd_occupancy<TW, TH, BATCH, true>() : fwd_occupancy<TW, TH, BATCH, false>();
+  const long long grid = (long long)num_sms * occ;
   return grid > n_tiles ? n_tiles : grid;
 }
 
@@ -550,9 +609,9 @@ void launch_forward_instance(const ViewDev* views, int n_views, long long n_tile
                              const int* order, float* image, float* T, unsigned* last, unsigned* gp, float4* ckpt,
                              unsigned* cmask, int* chunk_tile, int* tile_chunks, unsigned* tile_done, int num_sms,
                              cudaStream_t s) {
-  launch_dep(k_blend_forward<TW, TH, BATCH>, dim3((unsigned)forward_grid<TW, TH, BATCH>(n_tiles, num_sms)),
-      dim3(TW * TH), 0, s, views, n_views, n_tiles, ranges, vals, pb, sp, ctl, order, image, T, last, gp, ckpt, cmask,
-      chunk_tile, tile_chunks, tile_done);
+  launch_dep(few_tiles(n_tiles, num_sms) ? k_blend_forward_few<TW, TH, BATCH> : k_blend_forward<TW, TH, BATCH>,
+      dim3((unsigned)forward_grid<TW, TH, BATCH>(n_tiles, num_sms)), dim3(TW * TH), 0, s, views, n_views, n_tiles,
+      ranges, vals, pb, sp, ctl, order, image, T, last, gp, ckpt, cmask, chunk_tile, tile_chunks, tile_done);
 }
 }  // namespace
 

@@ -80,6 +80,29 @@ def test_walk_edges(n, opacity, size):
     ras.close()
 
 
+def test_few_and_many_tiles_agree():
+    """A picture small enough for the four-candidate walk and the same picture with a margin that takes the
+    tile count past the line: the pixels both have are the same bits."""
+    import torch
+    import paper_2503_13086_gb300 as gs
+    p = gi.cube_scene(6000, seed=9, logscale=(-3.5, 0.6))
+    small = gi.identity_camera(200, 120, 150.0)
+    big = dict(small, width=200 + 16 * 60, height=120 + 16 * 60)  # 13 x 8 and 73 x 68 tiles, the same origin
+    # (the focal-plane clamp depends on the image size: keep it out of play)
+    keep = np.abs(p[0, :6000] / p[2, :6000]) < 0.6
+    p[10, :6000][~keep] = -20.0
+    p[10, :6000][np.abs(p[1, :6000] / p[2, :6000]) > 0.4] = -20.0
+    P = torch.tensor(p, device="cuda")
+    ras = gs.Raster()
+    a = ras.forward(P, 6000, [small])
+    a = {k: a[k].cpu().numpy() for k in ("image", "T", "gp")}
+    b = ras.forward(P, 6000, [big])
+    assert np.array_equal(a["image"].reshape(3, 120, 200), b["image"].cpu().numpy().reshape(3, 1080, 1160)[:, :120, :200])
+    assert np.array_equal(a["T"].reshape(120, 200), b["T"].cpu().numpy().reshape(1080, 1160)[:120, :200])
+    assert np.array_equal(a["gp"].reshape(120, 200), b["gp"].cpu().numpy().reshape(1080, 1160)[:120, :200])
+    ras.close()
+
+
 @pytest.mark.parametrize("load", [0.0, 0.4])
 @pytest.mark.parametrize("tile", [(16, 16, 256), (32, 8, 256), (16, 8, 256)])
 def test_backward_item_sharing(tile, load):
