@@ -398,11 +398,11 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
     mark(s, 4);
     mark(s, 5);
   } else if (list_built) {
+    mark(s, 3);  // (emission and sorts timed together, as the sort)
     launch_sort_large(proj(), vd(), stride, n_items, static_cast<unsigned long long*>(list0.p),
                       static_cast<unsigned long long*>(list1.p), static_cast<unsigned*>(place_of.p), list_state(1), k0, k1,
                       v0, static_cast<unsigned*>(inst_rec.p), hist(), sort_state(), tile_bits, (long long)m_cap, num_sms,
                       ctl(), s);
-    mark(s, 3);  // (emission and sorts timed together, as the sort)
     mark(s, 4);
     launch_ranges(k0, ranges(), tile_bits, 32, (long long)m_cap, ctl(), s);
     launch_tile_order(ranges(), n_tiles, static_cast<int*>(order.p), ctl(), s);
