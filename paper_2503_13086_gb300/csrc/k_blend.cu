@@ -13,8 +13,8 @@
 // a job ahead of the tile's slowest block instead of waiting for it at a CTA barrier.  Jobs are
 // walked in chunks of 32.  A warp skips a Gaussian outright when the bounding box of its 1/255 cutoff
 // ellipse misses the warp's block (warp-uniform).  The others are taken two at a time (four when the tiles
-// are few, see few_tiles) without a branch: every lane evaluates both exponents and alphas, then blends them in list order under predicates.  A
-// pixel's walk is one dependent chain, and the longest lists set the kernel's duration from a few
+// are few, see few_tiles) without a branch: every lane evaluates their exponents and alphas, then blends
+// them in list order under predicates.  A pixel's walk is one dependent chain, and the longest lists set the kernel's duration from a few
 // thousand Gaussians up, so what counts is the chain's length per candidate: with a branch per test
 // (cutoff, alpha, stop) it was about 300 cycles, in this form about 210 when a CTA has its SM to itself,
 // and about 48 instead of 62 instructions.  A stopped pixel's x becomes NaN, which fails every later
@@ -458,7 +458,7 @@ __device__ __forceinline__ void blend_forward(
       }
       if (jg0 > 0 && !done) ckpt[at] = make_float4(T, C0, C1, C2);
       unsigned mask = 0u;
-      // One straight line per candidate, two candidates in flight: every lane evaluates both
+      // One straight line per candidate, DEEP candidates in flight: every lane evaluates their
       // exponents and alphas, then they are blended in list order under predicates.
       if (DEEP > 2) {
         while (cand) {
@@ -586,11 +586,12 @@ void init_forward_instance() {
 }
 
 // With few tiles the longest lists' chains are the kernel's duration and most of the chip idles, so four
-// candidates go into each round of the walk at 128 registers and two CTAs per SM (per candidate about 130
-// instead of 210 cycles).  Up to 16 tiles per SM: 616 -> 452 us on a 128 x 96 image of 150k Gaussians (48
-// tiles), 164 -> 133 at 300 x 200 of 120k (247), 110 -> 84 at 160 x 120 of 30k, 32 -> 26 at 128 x 97 of 3k, 70 -> 57 at
-// 640 x 360 of 60k (920), 91 -> 75 at 1000 x 600 of 200k (2394), 61 -> 62 at 960 x 540 of 60k (2040).  With 4346
-// tiles it depends on the lists, which the host does not know (262 against 330 us at 1.9M, but 123 against
+// candidates go into each round of the walk at 108 registers and two 256-thread CTAs per SM (per candidate
+// about 130 instead of 210 cycles).  Up to 16 tiles (of 16 x 16) per SM: 616 -> 452 us on a 128 x 96 image of
+// 150k Gaussians (48 tiles), 110 -> 84 at 160 x 120 of 30k (80), 164 -> 133 at 300 x 200 of 120k (247), 32 -> 26
+// at 128 x 97 of 3k, 70 -> 57 at 640 x 360 of 60k (920), 61 -> 62 at 960 x 540 of 60k (2040), 91 -> 75 at
+// 1000 x 600 of 200k (2394).  Smaller tiles have shorter lists for the same count and stay under the line
+// only on smaller images.  With 4346 tiles it depends on the lists, which the host does not know (262 against 330 us at 1.9M, but 123 against
 // 110 at 200k with large Gaussians over the image), and with 8160 and more the lost occupancy shows (148
 // against 118, 1042 against 751 on nine views).  Eight per round: 471 us on the 48 tiles.
 bool few_tiles(long long n_tiles, int num_sms) { return n_tiles <= 16ll * num_sms; }
