@@ -673,6 +673,7 @@ __device__ __forceinline__ float fast_rcp(float x) {
 }
 
 constexpr int kBwdWarps = 4;
+constexpr unsigned kClaimWords = 2;  // per pair of warps that share an item
 constexpr int kGroup = 3;  // Gaussians whose gradient terms are summed together (3 x 9 <= 32 lanes)
 constexpr int kBwdPairs = 2;  // packed pixel pairs per lane (4 pixels, 128 per round)
 
@@ -722,13 +723,17 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) k_blend_backward(
   const unsigned lt = (1u << lane) - 1u;
   const int part = SPLIT ? warp & 1 : 0;
   const auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp >> 1)) : "memory"); };
-  __shared__ unsigned s_claim[kBwdWarps / 2];
-  for (;;) {
+  // A pair's claims alternate between two words: an id without a chunk sends both warps straight to the next
+  // claim, so the even warp may store that one before the odd warp has read this one.  The store after it,
+  // to this word again, lies behind the next turn's barrier, which the odd warp reaches only after its read.
+  __shared__ unsigned s_claim[kBwdWarps / 2][kClaimWords];
+  for (unsigned turn = 0;; ++turn) {
     long long id = 0;
     if (SPLIT) {
-      if (part == 0 && lane == 0) s_claim[warp >> 1] = atomicAdd(&ctl->bwd_work, 1u);
+      unsigned* claim = &s_claim[warp >> 1][turn % kClaimWords];
+      if (part == 0 && lane == 0) *claim = atomicAdd(&ctl->bwd_work, 1u);
       pair_sync();  // (also: the even warp is through with the odd one's sums)
-      id = (long long)s_claim[warp >> 1];
+      id = (long long)*claim;
     } else {
       if (lane == 0) id = (long long)atomicAdd(&ctl->bwd_work, 1u);
       id = __shfl_sync(0xffffffffu, id, 0);
