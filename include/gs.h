@@ -461,7 +461,7 @@ GS_API gs_status gs_autotune_clear(void);
 /* The two inter-CTA waits of a step (the decoupled look-back of the K2 scan and of each K4 sort
  * pass) spin a bounded number of times; a wait that gives up sets an error bit in the step's
  * control block and its CTA finishes its work with the prefix it has, so the kernel returns and the
- * context stays usable, and the step reports GS_ERR_TIMEOUT.  This call runs each wait once on a
+ * context stays usable; the step's later kernels return at once, and it reports GS_ERR_TIMEOUT.  This call runs each wait once on a
  * two-tile problem by a single CTA that holds the second tile: the first tile is never started,
  * so the wait can only end by giving up.
  *   spin_limit  rounds of the look-back before giving up; 0 = the limit the steps use
@@ -484,6 +484,14 @@ GS_API gs_status gs_wait_probe(uint32_t spin_limit, uint32_t out_error[2], float
  * Synchronous.  Allocates about 90 KB of device memory and frees it before returning.  Returns
  * GS_OK when the run completed (whatever it reports), GS_ERR_CUDA otherwise. */
 GS_API gs_status gs_loss_wait_probe(uint32_t spin_limit, uint32_t* out_error, float* out_ms);
+
+/* Host-side fault injection for what follows a wait that gave up: the next forward of the rasterizer (the
+ * next step, render or autotuning pass of the session) starts with the error bit already set.  Its
+ * kernels after the scan then write nothing and the call reports GS_ERR_TIMEOUT (a forward without
+ * out_pairs: the backward after it); a session's Gaussians, moments and counters stay as they were, and
+ * the call after it runs as usual.  Host only; returns GS_ERR_INVALID_ARG for NULL. */
+GS_API gs_status gs_raster_time_out_next(gs_raster* r);
+GS_API gs_status gs_field_time_out_next(gs_field* f);
 
 /* ----------------------------------------------------------------------------------------
  * Allocation-free entry point.  The paper has no counterpart: this is a deployment variant.

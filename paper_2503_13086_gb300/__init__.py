@@ -165,6 +165,8 @@ SYMBOLS = {
     "gs_wait_probe": ([ctypes.c_uint32, P, P], I32),
     "gs_loss_wait_probe": ([ctypes.c_uint32, P, P], I32),
     "gs_field_corrupt_guard": ([P, I32, P, I32], I32),
+    "gs_raster_time_out_next": ([P], I32),
+    "gs_field_time_out_next": ([P], I32),
     "gs_schedule_plan": ([P, P, P, I32, I32, P, P, P, P, P, P], I32),
 }
 
@@ -319,6 +321,10 @@ class Raster:
 
     def set_timing(self, on=True):
         _check(self._lib.gs_raster_set_timing(self._h, 1 if on else 0))
+
+    def time_out_next(self):
+        """The next forward behaves as if one of its bounded waits had given up (failure detection)."""
+        _check(self._lib.gs_raster_time_out_next(self._h))
 
     def kernel_times(self):
         out = (ctypes.c_float * 9)()
@@ -570,6 +576,10 @@ class Field:
         _check(self._lib.gs_field_densify_stats(self._h, a.ctypes.data_as(ctypes.c_void_p),
                                                 c.ctypes.data_as(ctypes.c_void_p)))
         return a[:n], c[:n]
+
+    def time_out_next(self):
+        """The next step, render or autotuning pass behaves as if one of its bounded waits had given up."""
+        _check(self._lib.gs_field_time_out_next(self._h))
 
     def corrupt_guard(self, index):
         """Overwrite one guard word behind the index-th allocated device buffer of the session (host-side

@@ -74,7 +74,7 @@ struct Control {
   unsigned long long gp_pixels; // pixels with G_p > 0 (the "visible range" of Eq. 9)
   unsigned long long gp_sq;     // sum of G_p^2 over those pixels
   unsigned int overflow;        // instance capacity exceeded
-  unsigned int error;           // kErr* bits
+  unsigned int error;           // kErr* bits; once set, the kernels after the scan do nothing (step_void)
   unsigned int dmax;            // largest fp32 depth bits of a record with instances
   unsigned int dnot;            // ~ smallest such bits (so that the cleared 0 is neutral)
   unsigned int scan_ticket;
@@ -155,8 +155,15 @@ __device__ __forceinline__ KeyLayout key_layout(const Control* ctl, int tile_bit
   return k;
 }
 
+// Whether the rest of the step has nothing to do: its instances overflow the buffers (kErrOverflow), or a
+// bounded wait gave up (kErrTimeout).  After the latter offsets, lists and counts are not to be relied on:
+// a stale list word holds any record or digit, and a store through it may fall outside its buffer.
+// A kernel whose own waits may set the bit asks once per CTA (its threads could see different answers).
+__device__ __forceinline__ bool step_void(const Control* ctl) { return ctl->error != 0u; }
+
 // Bounded spin limit for inter-CTA waits (decoupled look-back).  On expiry the waiting CTA sets
-// kErrTimeout and proceeds; the host reports GS_ERR_TIMEOUT.  A round of the scan's look-back takes
+// kErrTimeout and finishes its own work (in range: its offsets come out too small, never too large), the
+// kernels after it return at once, and the host reports GS_ERR_TIMEOUT.  A round of the scan's look-back takes
 // about 0.29 us on a GB300 and one of a sort pass's about 0.37 us, so a wait that nothing ends gives
 // up after about 1.2 / 1.6 s; a predecessor that is running publishes within microseconds.
 constexpr unsigned kSpinLimit = 1u << 22;

@@ -98,6 +98,7 @@ struct Raster {
   DevBuf ledger_d;  // Ledger of the current run of steps
   DevBuf own_image, own_last, own_dimage;  // used by sessions
   unsigned long long m_cap = 0;
+  bool time_out_next = false;  // the next step starts with a wait already given up (failure detection)
   bool sized_before = false;  // m_cap comes from an instance count read back at least once
   size_t bytes_in_use = 0;
 

@@ -644,7 +644,7 @@ struct Field {
       sized_tiling = R.tiling;
       return GS_OK;
     }
-    if (!cfg.use_graph) return enqueue_step(false);
+    if (!cfg.use_graph || R.time_out_next) return enqueue_step(false);
     GraphKey key{cur_sizes, signature()};
     GraphEntry* ge = nullptr;
     for (auto& g : graphs)
@@ -859,14 +859,14 @@ struct Field {
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("step launch: ") + cudaGetErrorString(e));
     const Ledger& Lg = *R.ledger_h;
-    if (Lg.error & kErrTimeout) return fail(GS_ERR_TIMEOUT, "a device-side wait (decoupled look-back) timed out");
-    if (cfg.debug_canaries && (s = check_guard_words())) return s;
+    if (!(Lg.error & kErrTimeout) && cfg.debug_canaries && (s = check_guard_words())) return s;
     const size_t ok = std::min<size_t>(Lg.steps_ok, count);
-    // commit the completed prefix only
+    // commit the completed prefix only (a step in which a wait gave up, and those after it, changed nothing)
     adam_step = step0 + (long long)ok;
     for (size_t j = 0; j < images.size(); ++j) images[j].T = j < T0.size() ? T0[j] : 0;
     for (size_t k = 0; k < ok; ++k)
       for (int id : groups[first_group + k]) images[id].T += 1;
+    if (Lg.error & kErrTimeout) return fail(GS_ERR_TIMEOUT, "a device-side wait (decoupled look-back) timed out");
     if (ok < count) {
       // a step overflowed the instance buffers: grow them for the next try
       if ((s = R.ensure_instances(Lg.m_need + Lg.m_need / 4 + 1024))) return s;
@@ -1354,6 +1354,12 @@ gs_status gs_field_densify_stats(gs_field* ff, float* host_sum, float* host_coun
   if (f->n > 0 && host_count &&
       cudaMemcpy(host_count, d + f->stride, (size_t)f->n * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(GS_ERR_CUDA, "reading the statistics failed");
+  return GS_OK;
+}
+
+gs_status gs_field_time_out_next(gs_field* ff) {
+  if (!ff) return fail(GS_ERR_INVALID_ARG, "NULL field");
+  F(ff)->r->time_out_next = true;
   return GS_OK;
 }
 

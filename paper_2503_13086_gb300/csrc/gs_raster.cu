@@ -354,6 +354,8 @@ gs_status Raster::upload(cudaStream_t s) {
 
 gs_status Raster::enqueue_forward_head(cudaStream_t s, const float* params, int stride_, bool size_exactly) {
   cudaMemsetAsync(zeroA.p, 0, zeroA_bytes, s);
+  if (time_out_next) cudaMemsetAsync(&ctl()->error, (int)kErrTimeout, 1, s);  // (the lowest byte)
+  time_out_next = false;
   // zeroB is cleared here too unless the sizing below may reallocate it, so that the kernels from
   // K1 on follow one another with no other node between them (programmatic dependent launch)
   zeroB_pending = size_exactly;
@@ -587,6 +589,7 @@ gs_status gs_raster_loss(gs_raster* rr, void* stream, const float* image, const 
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("loss: ") + cudaGetErrorString(e));
     *out_loss = r->ctl_h->loss;
+    return r->check_control();
   }
   return GS_OK;
 }
@@ -727,6 +730,12 @@ gs_status gs_raster_set_tiling(gs_raster* rr, const gs_tiling* t) {
   const gs::Tiling tl{t->tile_w, t->tile_h, t->batch};
   if (!gs::tiling_supported(tl)) return fail(GS_ERR_INVALID_ARG, "tiling not among gs_tiling_candidates");
   r->tiling = tl;
+  return GS_OK;
+}
+
+gs_status gs_raster_time_out_next(gs_raster* rr) {
+  if (!rr) return fail(GS_ERR_INVALID_ARG, "NULL raster");
+  reinterpret_cast<gs::Raster*>(rr)->time_out_next = true;
   return GS_OK;
 }
 

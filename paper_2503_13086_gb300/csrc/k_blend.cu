@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint2* __restrict__ r
   dep_release();
   __shared__ unsigned s_cnt[32];
   __shared__ unsigned s_base[32];
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   if (threadIdx.x < 32) s_cnt[threadIdx.x] = 0u;
   __syncthreads();
   for (long long t = threadIdx.x; t < n_tiles; t += blockDim.x) {
@@ -200,7 +200,6 @@ __device__ __forceinline__ void blend_forward(
   __shared__ long long s_cur_t;
   __shared__ unsigned s_cur_start;
   __shared__ int s_cur_L, s_cur_nb, s_cur_seq;
-  if (ctl->overflow) return;
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const float bg0 = sp->bg[0], bg1 = sp->bg[1], bg2 = sp->bg[2];
@@ -319,7 +318,7 @@ __device__ __forceinline__ void blend_forward(
     for (int b = 0; b < 4; ++b) s_fin[b] = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
+  if (__syncthreads_or(tid == 0 && step_void(ctl))) return;
   bool ok = warp != 0 || stage(0);
 
   // this thread's pixel of the current tile
@@ -702,7 +701,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) k_blend_backward(
   using Sh = Shape<TW, TH>;
   constexpr int kPix = Sh::kPix;
   BwdWarp<kPix>& S = reinterpret_cast<BwdWarp<kPix>*>(smem_raw)[warp];
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   // Eq. 9-10: dL/dG_p = lambda_load (G_p - mean) / (N std) over the N pixels with G_p > 0 (K6's
   // moments of all the step's views); it reaches alpha through the soft count, the sum of the
   // blended Gaussians' alphas.  load_a = lambda_load / (N std), load_mu = mean; off without G_p.

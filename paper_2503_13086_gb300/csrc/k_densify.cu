@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(256) k_densify_stats(int n, int stride, int n_
   dep_wait();
   dep_release();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || ctl->overflow) return;
+  if (i >= n || step_void(ctl)) return;
   const long long n_rec = (long long)n_views * stride;
   float acc = dstat[i], cnt = dstat[stride + i];
   for (int v = 0; v < n_views; ++v) {

@@ -179,7 +179,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
   LossFwdSmem& S = *reinterpret_cast<LossFwdSmem*>(smem_raw);
   __shared__ double s_red[2][8];
   __shared__ bool s_last;
-  if (ld_relaxed_u32(&ctl->overflow)) return;
+  // (step_void, read through L2: the blend forward may still be running and set the bit)
+  if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(&ctl->error) != 0u)) {
+    if (threadIdx.x == 0 && ledger) atomicOr(&ledger->error, ld_relaxed_u32(&ctl->error) & kErrTimeout);
+    return;
+  }
   const long long b = blockIdx.x;
   const int v = view_of_block(views, n_views, b);
   const ViewDev& V = views[v];
@@ -382,8 +386,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
       ledger->pairs += pairs;
       ledger->blended += blended;
       ledger->instances += ld_relaxed_u64(&ctl->m_total);
-      ledger->steps_ok += 1u;
-      ledger->error |= ld_relaxed_u32(&ctl->error);
+      const unsigned err = ld_relaxed_u32(&ctl->error);
+      ledger->steps_ok += err ? 0u : 1u;
+      ledger->error |= err;
       ledger->last_gp_sum = blended;
       ledger->last_gp_pixels = gp_pixels;
       ledger->last_gp_sq = gp_sq;
@@ -401,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_backward(const ViewDev* __
   dep_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   LossBwdSmem& S = *reinterpret_cast<LossBwdSmem*>(smem_raw);
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   const long long b = blockIdx.x;
   const int v = view_of_block(views, n_views, b);
   const ViewDev& V = views[v];

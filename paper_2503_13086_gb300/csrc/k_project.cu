@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) k_inst_reduce(const unsigned* __restrict_
                                                      float* __restrict__ tail) {
   dep_wait();
   dep_release();
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   const int lane = threadIdx.x & 31;
   const unsigned long long M = ctl->m_total;
   const unsigned long long n_chunks = (M + 31) >> 5;
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(256) k_inst_carry(const unsigned* __restrict__
   dep_wait();
   dep_release();
   __shared__ float s_head[8][9 * 32];
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // four runs of eight records (whole 32-byte sectors), a quarter of all records apart: the large records
   // of an arrival lie next to each other, and one warp should not get 32 of them
@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(256, 2) k_project_backward(
   dep_release();
   const long long n_rec = (long long)n_views * stride;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ctl->overflow) return;  // the step was skipped; the host re-runs it with more capacity
+  if (step_void(ctl)) return;  // the step was skipped; the host re-runs it with more capacity
   const bool unseen = vec_ok && warp_unseen(count, n_views, stride, i, sp->n);
   if (i >= sp->n) return;
 
@@ -917,7 +917,7 @@ __global__ void __launch_bounds__(256, 2) k_project_backward_views(
   const long long n_rec = (long long)n_views * stride;
   __shared__ float s_gsh[48 * 256];  // [row][thread]
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   const bool unseen = vec_ok && warp_unseen(count, n_views, stride, i, sp->n);
   if (i >= sp->n) return;
   float* gsh = s_gsh + threadIdx.x;

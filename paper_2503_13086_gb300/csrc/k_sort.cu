@@ -101,11 +101,9 @@ __global__ void __launch_bounds__(MODE == SCAN_COMPACT ? kLargeScanThreads : kSc
   __shared__ unsigned s_warp[kThr / 32], s_lwarp[kThr / 32];
   __shared__ unsigned long long s_excl;
   __shared__ unsigned s_lexcl;
-  if (MODE == SCAN_LIST) {
-    if (ctl->overflow) return;
-    n_items = (long long)ctl->listed;
-  }
-  if (threadIdx.x == 0) s_tile = atomicAdd(MODE == SCAN_LIST ? &ctl->list_ticket : &ctl->scan_ticket, 1u);
+  if (MODE == SCAN_LIST) n_items = (long long)ctl->listed;
+  if (threadIdx.x == 0)
+    s_tile = MODE == SCAN_LIST ? (step_void(ctl) ? ~0u : atomicAdd(&ctl->list_ticket, 1u)) : atomicAdd(&ctl->scan_ticket, 1u);
   __syncthreads();
   const unsigned tile = s_tile;
   const long long num_tiles = (n_items + kTileItems - 1) / kTileItems;
@@ -188,8 +186,8 @@ __global__ void __launch_bounds__(MODE == SCAN_COMPACT ? kLargeScanThreads : kSc
       if (MODE != SCAN_LIST && (long long)tile == num_tiles - 1) {
         const unsigned long long m = excl + total;
         ctl->m_total = m;
-        // an overflow skips this step; an earlier skipped step of the run skips it too
-        if (m > m_cap || (ledger && ledger->skip)) {
+        // an overflow skips this step; an earlier skipped or timed-out step of the run skips it too
+        if (m > m_cap || (ledger && (ledger->skip || ledger->error))) {
           ctl->overflow = 1u;
           atomicOr(&ctl->error, kErrOverflow);
           if (ledger) {
@@ -261,7 +259,7 @@ __global__ void __launch_bounds__(256) k_fill_owner(const unsigned* __restrict__
                                                     unsigned* __restrict__ inst_rec, const Control* __restrict__ ctl) {
   dep_wait();
   dep_release();
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   const int lane = threadIdx.x & 31;
   const long long rec = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned cnt = rec < n_items ? count[rec] : 0u;
@@ -296,7 +294,7 @@ __global__ void __launch_bounds__(1024) k_emit(const ProjBuffers pb, const ViewD
   const int depth_passes = min(passes, kl.D / kSortBits);
   unsigned long long* __restrict__ keys = (passes & 1) ? keys1 : keys0;
   unsigned* __restrict__ vals = (passes & 1) ? vals1 : vals0;
-  if (!ctl->overflow) {
+  if (!step_void(ctl)) {
     const unsigned long long M = ctl->m_total;
     for (unsigned long long e = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; e < M;
          e += (unsigned long long)gridDim.x * blockDim.x) {
@@ -425,7 +423,7 @@ __global__ void __launch_bounds__(kSortThreads, kSortMinBlocks) k_sort_pass(unsi
   unsigned long long* __restrict__ kout = from1 ? keys0 : keys1;
   unsigned* __restrict__ vout = from1 ? vals0 : vals1;
   const unsigned long long M = ctl->m_total;
-  if (threadIdx.x == 0) S.tile = atomicAdd(&ctl->sort_ticket[pass], 1u);
+  if (threadIdx.x == 0) S.tile = step_void(ctl) ? ~0u : atomicAdd(&ctl->sort_ticket[pass], 1u);
   for (int k = threadIdx.x; k < (kSortThreads / 32) * kSortBins; k += kSortThreads) {
     (&S.cnt[0][0])[k] = 0u;
     (&S.mask[0][0])[k] = 0u;
@@ -574,7 +572,7 @@ __global__ void __launch_bounds__(kSortThreads, kWordMinBlocks) k_sort_pass_word
   WordSmem& S = *reinterpret_cast<WordSmem*>(smem_raw);
   if (ctl->overflow) return;
   const unsigned long long M = by_record ? (unsigned long long)ctl->listed : ctl->m_total;
-  if (threadIdx.x == 0) S.tile = atomicAdd(&ctl->sort_ticket[ticket], 1u);
+  if (threadIdx.x == 0) S.tile = step_void(ctl) ? ~0u : atomicAdd(&ctl->sort_ticket[ticket], 1u);
   for (int k = threadIdx.x; k < (kSortThreads / 32) * kSortBins; k += kSortThreads) {
     (&S.cnt[0][0])[k] = 0u;
     (&S.mask[0][0])[k] = 0u;
@@ -676,7 +674,7 @@ __global__ void __launch_bounds__(1024) k_depth_hist(const unsigned long long* _
   dep_wait();
   dep_release();
   __shared__ unsigned s_hist[kDepthPasses][kSortBins];
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   for (int k = threadIdx.x; k < kDepthPasses * kSortBins; k += blockDim.x) (&s_hist[0][0])[k] = 0u;
   __syncthreads();
   const unsigned n = ctl->listed;
@@ -701,7 +699,7 @@ __global__ void __launch_bounds__(512) k_emit_words(const ProjBuffers pb, const 
   dep_wait();
   dep_release();
   __shared__ unsigned s_hist[kMaxSortPasses - kDepthPasses][kSortBins];
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   for (int k = threadIdx.x; k < tile_passes * kSortBins; k += blockDim.x) (&s_hist[0][0])[k] = 0u;
   __syncthreads();
   const unsigned long long M = ctl->m_total;
@@ -773,7 +771,7 @@ __global__ void __launch_bounds__(256) k_ranges(const unsigned long long* __rest
                                                 int tile_bits, int shift, const Control* __restrict__ ctl) {
   dep_wait();
   dep_release();
-  if (ctl->overflow) return;
+  if (step_void(ctl)) return;
   const unsigned long long M = ctl->m_total;
   const int D = shift ? shift : key_layout(ctl, tile_bits).D;  // where the tile starts in the key
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < M;
@@ -869,7 +867,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_bin_small(const ProjBuffer
   dep_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmallSmem& S = *reinterpret_cast<SmallSmem*>(smem_raw);
-  if (ctl->overflow) return;  // every CTA of the cluster alike
+  if (step_void(ctl)) return;  // every CTA of the cluster alike
   const unsigned M = (unsigned)ctl->m_total;
   const KeyLayout kl = key_layout(ctl, tile_bits);
   const unsigned r = cluster_rank(), C = cluster_size();
