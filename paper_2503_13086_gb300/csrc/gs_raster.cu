@@ -527,6 +527,9 @@ gs_status gs_raster_forward(gs_raster* rr, void* stream, const float* params, in
     return fail(GS_ERR_INVALID_ARG, "need 0 <= n <= stride, stride a positive multiple of 32");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   gs_status st;
+  // from here on the views, counts and lists of the forward before are overwritten: a forward that fails
+  // leaves nothing for a loss or a backward (they would index released buffers with its counts)
+  r->have_forward = false;
   if ((st = r->set_views(cams, n_views, nullptr))) return st;
   r->stride = (int)stride;
   r->n = (int)n;
@@ -549,10 +552,12 @@ gs_status gs_raster_forward(gs_raster* rr, void* stream, const float* params, in
     if ((st = r->enqueue_forward_head(s, params, (int)stride, sized))) return st;
     if ((st = r->ensure_instances(r->m_cap))) return st;
     if ((st = r->enqueue_forward_tail(s, out_image, out_T, out_last, out_gp, false))) return st;
-    r->have_forward = true;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("forward launch: ") + cudaGetErrorString(e));
-    if (!out_pairs) return GS_OK;
+    if (!out_pairs) {
+      r->have_forward = true;
+      return GS_OK;
+    }
     r->enqueue_readback(s);
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("forward: ") + cudaGetErrorString(e));
@@ -560,7 +565,9 @@ gs_status gs_raster_forward(gs_raster* rr, void* stream, const float* params, in
     sized = true;
   }
   *out_pairs = r->ctl_h->pairs;
-  return r->check_control();
+  st = r->check_control();
+  r->have_forward = st == GS_OK;
+  return st;
 }
 
 gs_status gs_raster_loss(gs_raster* rr, void* stream, const float* image, const float* target,
