@@ -429,7 +429,7 @@ GS_API gs_status gs_field_kernel_times(gs_field* f, float out_ms[9], int64_t* ou
 
 /* Autotuner of the tile shape and blend batch (the paper gives none; see gs_tiling).  Times every
  * compiled candidate on the field's current state and the given views (host array, 1..32 image
- * ids): one sizing pass, one warm-up, then `reps` (>= 1) back-to-back runs of a whole step --
+ * ids): one sizing pass of each, then of each one warm-up and `reps` (>= 1) back-to-back runs of a whole step --
  * projection, scan, key emission, sort, ranges, blend forward, loss, blend backward and the
  * projection backward -- except that the projection backward writes nothing (no Adam update,
  * which costs the same for every tiling), so the field's parameters, moments and T_j are
