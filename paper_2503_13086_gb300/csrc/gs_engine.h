@@ -92,7 +92,6 @@ struct Raster {
   bool zeroB_pending = true;  // zeroB still to be cleared by the forward tail
   DevBuf xyo, conic, rgb, depth, radius, rect, count, offsets, clamp, g2s;
   DevBuf keys0, keys1, vals0, vals1, ginst, ckpt, cmask, order, tile_chunks;
-  DevBuf list0, list1, place_of;  // large steps: listed records (two buffers), where each one's instances go
   DevBuf inst_rec, carry;  // instance -> record, K9a partials
   DevBuf partials, block_sums;
   DevBuf ledger_d;  // Ledger of the current run of steps
@@ -122,7 +121,6 @@ struct Raster {
   uint2* ranges() const;
   int* chunk_tile() const;
   unsigned* tile_done() const;  // per tile: 1 once the blend forward finished it
-  unsigned long long* list_state(int k) const;  // look-back states of the list (0) and of its count scan (1)
   // Large steps sort depth and tile apart (k_sort.cu).  Against the (tile, depth) passes, K2 - K4 together:
   // 529 -> 380 us at 6.5M instances of 2.0M listed records, 218 -> 201 at 2.8M of 0.86M, 159 -> 154 at 1.6M of
   // 0.5M, but 121 -> 130 at 1.2M and 114 -> 129 at 1.0M on a 160 x 100 image (one pass fewer without it), where
@@ -133,8 +131,18 @@ struct Raster {
     return n_rec >= kLargeRecords && n_rec < (1ll << 31) && tile_bits <= 8 * (kMaxSortPasses - kDepthPasses) &&
            (long long)m_cap >= kLargeInstances;
   }
-  bool list_ready = false;  // ensure_records made the list's buffers for the current views
-  bool list_built = false;  // the last forward head listed its records (not one whose m_cap grew after ensure_records)
+  // What the large path needs besides, all of it inside g2s: from the projection to the end of the sort the
+  // per-record gradients of the step before are no longer read and this step's not yet written.  So the
+  // path takes no memory of its own, and no call is refused for it.
+  struct LargeScratch {
+    unsigned long long *list0, *list1;  // listed records (two buffers)
+    unsigned* place_of;                 // per record: where its instances go
+    unsigned long long* scan_state[2];  // look-back states of the list and of the scan of its counts
+    unsigned* sort_state;               // and of the depth passes
+    size_t state_bytes;                 // of the three together (contiguous from scan_state[0], cleared by each step)
+  };
+  LargeScratch large_scratch() const;
+  bool list_built = false;  // the last forward head listed its records
   ProjBuffers proj() const;
   const StepParams* sp() const { return static_cast<const StepParams*>(sp_d.p); }
   const ViewDev* vd() const { return static_cast<const ViewDev*>(views_d.p); }

@@ -339,7 +339,7 @@ struct Field {
           {"clamp", &R.clamp}, {"g2s", &R.g2s}, {"keys0", &R.keys0}, {"keys1", &R.keys1}, {"vals0", &R.vals0},
           {"vals1", &R.vals1}, {"ginst", &R.ginst}, {"ckpt", &R.ckpt}, {"cmask", &R.cmask}, {"order", &R.order},
           {"tile_chunks", &R.tile_chunks}, {"inst_rec", &R.inst_rec}, {"carry", &R.carry},
-          {"listed records 0", &R.list0}, {"listed records 1", &R.list1}, {"instance places", &R.place_of}, {"partials", &R.partials},
+          {"partials", &R.partials},
           {"block_sums", &R.block_sums}, {"raster image", &R.own_image}, {"raster last", &R.own_last},
           {"raster dimage", &R.own_dimage}};
       v.insert(v.end(), std::begin(rr), std::end(rr));
@@ -434,7 +434,7 @@ struct Field {
     const DevBuf* bufs[] = {&params, &adam_m, &adam_v, &dstat, &step_img, &step_dimg, &step_last, &step_T, &step_gp,
                             &R.sp_d, &R.views_d, &R.zeroA, &R.zeroB, &R.xyo, &R.conic, &R.rgb, &R.depth, &R.radius,
                             &R.rect, &R.count, &R.offsets, &R.clamp, &R.g2s, &R.keys0, &R.keys1, &R.vals0, &R.vals1, &R.ginst,
-                            &R.inst_rec, &R.carry, &R.list0, &R.list1, &R.place_of,
+                            &R.inst_rec, &R.carry,
                             &R.ckpt, &R.cmask, &R.order, &R.tile_chunks, &R.partials, &R.block_sums};
     for (const DevBuf* b : bufs) v.push_back((unsigned long long)(uintptr_t)b->p);
     const unsigned long long lay[] = {(unsigned long long)stride, R.m_cap, (unsigned long long)(uintptr_t)R.dstat, (unsigned long long)R.passes,

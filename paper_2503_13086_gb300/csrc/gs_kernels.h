@@ -71,9 +71,9 @@ void launch_ranges(const unsigned long long* keys, uint2* ranges, int tile_bits,
 int word_tile_passes(int tile_bits);
 void launch_sort_large(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items,
                        unsigned long long* list0, unsigned long long* list1, unsigned* place_of,
-                       unsigned long long* list_state, unsigned long long* words0, unsigned long long* words1,
-                       unsigned* vals_out, unsigned* inst_rec, unsigned* hist, unsigned* state, int tile_bits,
-                       long long m_cap, int num_sms, Control* ctl, cudaStream_t s);
+                       unsigned long long* list_state, unsigned* depth_state, unsigned long long* words0,
+                       unsigned long long* words1, unsigned* vals_out, unsigned* inst_rec, unsigned* hist,
+                       unsigned* tile_state, int tile_bits, long long m_cap, int num_sms, Control* ctl, cudaStream_t s);
 
 // Small steps: owner fill, then emission, sort, ranges and tile order in one launch of a cluster of
 // `cluster` CTAs (bin_small_cluster(m_cap, tile_bits), 0: the step is not small).

@@ -162,7 +162,7 @@ Raster::Raster() {
 
 Raster::~Raster() {
   DevBuf* all[] = {&sp_d, &views_d, &ledger_d, &zeroA, &zeroB, &xyo, &conic, &rgb, &depth, &radius, &rect, &count, &offsets,
-                   &clamp, &g2s, &keys0, &keys1, &vals0, &vals1, &ginst, &inst_rec, &carry, &list0, &list1, &place_of, &ckpt, &cmask, &order, &tile_chunks, &partials, &block_sums, &own_image,
+                   &clamp, &g2s, &keys0, &keys1, &vals0, &vals1, &ginst, &inst_rec, &carry, &ckpt, &cmask, &order, &tile_chunks, &partials, &block_sums, &own_image,
                    &own_last, &own_dimage};
   for (DevBuf* b : all) b->release(&bytes_in_use);
   if (sp_h) cudaFreeHost(sp_h);
@@ -177,9 +177,21 @@ Control* Raster::ctl() const { return reinterpret_cast<Control*>(zeroA.p); }
 unsigned long long* Raster::scan_state() const {
   return reinterpret_cast<unsigned long long*>(static_cast<char*>(zeroA.p) + kCtlBytes);
 }
-unsigned long long* Raster::list_state(int k) const {
-  const long long tiles = ((long long)n_views * stride + kScanTile - 1) / kScanTile;
-  return scan_state() + (size_t)(1 + k) * tiles;
+Raster::LargeScratch Raster::large_scratch() const {
+  const size_t recs = (size_t)n_views * stride;  // a multiple of 32
+  const size_t scan_tiles = (recs + kScanTile - 1) / kScanTile, sort_tiles = (recs + kSortTile - 1) / kSortTile;
+  static_assert(kDepthPasses * kSortBins * 4 <= kSortTile, "at most a byte per record and a last tile's");
+  static_assert(22 * kLargeRecords + kSortTile + 16 <= 36 * kLargeRecords, "the lists' 20 bytes and the states fit g2s");
+  LargeScratch L;
+  char* base = static_cast<char*>(g2s.p);
+  L.list0 = reinterpret_cast<unsigned long long*>(base);
+  L.list1 = L.list0 + recs;
+  L.place_of = reinterpret_cast<unsigned*>(L.list1 + recs);
+  L.scan_state[0] = reinterpret_cast<unsigned long long*>(L.place_of + recs);
+  L.scan_state[1] = L.scan_state[0] + scan_tiles;
+  L.sort_state = reinterpret_cast<unsigned*>(L.scan_state[1] + scan_tiles);
+  L.state_bytes = 2 * scan_tiles * 8 + (size_t)kDepthPasses * sort_tiles * kSortBins * 4;
+  return L;
 }
 unsigned* Raster::hist() const { return reinterpret_cast<unsigned*>(zeroB.p); }
 unsigned* Raster::sort_state() const {
@@ -264,15 +276,8 @@ gs_status Raster::ensure_records(int stride_) {
       (s = clamp.reserve(recs, &bytes_in_use)) || (s = g2s.reserve(recs * 36, &bytes_in_use)))
     return s;
   const long long scan_tiles = (recs + kScanTile - 1) / kScanTile;
-  stride = stride_;
-  list_ready = false;
-  const long long states = large() ? 3 : 1;
-  if ((s = zeroA.reserve(kCtlBytes + states * scan_tiles * 8, &bytes_in_use))) return s;
-  zeroA_bytes = kCtlBytes + states * scan_tiles * 8;
-  if (large() && ((s = list0.reserve(recs * 8, &bytes_in_use)) || (s = list1.reserve(recs * 8, &bytes_in_use)) ||
-                  (s = place_of.reserve(recs * 4, &bytes_in_use))))
-    return s;
-  list_ready = large();
+  if ((s = zeroA.reserve(kCtlBytes + scan_tiles * 8, &bytes_in_use))) return s;
+  zeroA_bytes = kCtlBytes + scan_tiles * 8;
   if ((s = partials.reserve(n_pix * 10 * 4, &bytes_in_use)) || (s = block_sums.reserve(n_loss_blocks * 16 * (n_loss_blocks <= loss_split_blocks(num_sms) ? 3 : 1), &bytes_in_use)))
     return s;
   return GS_OK;
@@ -307,12 +312,6 @@ gs_status Raster::ensure_instances(unsigned long long m) {
     return s;
   const unsigned long long sort_tiles = (m_cap + kSortTile - 1) / kSortTile;
   sort_state_bytes = (size_t)passes * sort_tiles * kSortBins * 4;
-  if (large()) {
-    const unsigned long long rec_tiles = ((unsigned long long)n_views * stride + kSortTile - 1) / kSortTile;
-    sort_state_bytes = std::max<size_t>(
-        sort_state_bytes,
-        ((size_t)kDepthPasses * rec_tiles + (size_t)word_tile_passes(tile_bits) * sort_tiles) * kSortBins * 4);
-  }
   ranges_bytes = (size_t)n_tiles * 8;
   chunk_bytes = (size_t)n_ids * 4;
   zeroB_bytes = kHistBytes + sort_state_bytes + ranges_bytes + chunk_bytes + (size_t)n_tiles * 4;
@@ -360,14 +359,15 @@ gs_status Raster::enqueue_forward_head(cudaStream_t s, const float* params, int 
   // K1 on follow one another with no other node between them (programmatic dependent launch)
   zeroB_pending = size_exactly;
   if (!size_exactly) cudaMemsetAsync(zeroB.p, 0, zeroB_bytes, s);
+  list_built = large();
+  const LargeScratch L = list_built ? large_scratch() : LargeScratch{};
+  if (list_built) cudaMemsetAsync(L.scan_state[0], 0, L.state_bytes, s);
   mark(s, 0);
   launch_project(params, stride_, n_views, sp(), vd(), proj(), s);
   mark(s, 1);
   const long long n_items = (long long)n_views * stride_;
-  list_built = list_ready;
   launch_scan(proj().count, proj().offsets, n_items, scan_state(), ctl(), size_exactly ? ~0ull : m_cap, ledger(), s,
-              proj().depth, list_built ? static_cast<unsigned long long*>(list0.p) : nullptr,
-              list_built ? list_state(0) : nullptr);
+              proj().depth, L.list0, L.scan_state[0]);
   mark(s, 2);
   if (size_exactly) {
     cudaMemcpyAsync(ctl_h, ctl(), sizeof(Control), cudaMemcpyDeviceToHost, s);
@@ -401,8 +401,8 @@ gs_status Raster::enqueue_forward_tail(cudaStream_t s, float* image, float* T, u
     mark(s, 5);
   } else if (list_built) {
     mark(s, 3);  // (emission and sorts timed together, as the sort)
-    launch_sort_large(proj(), vd(), stride, n_items, static_cast<unsigned long long*>(list0.p),
-                      static_cast<unsigned long long*>(list1.p), static_cast<unsigned*>(place_of.p), list_state(1), k0, k1,
+    const LargeScratch L = large_scratch();
+    launch_sort_large(proj(), vd(), stride, n_items, L.list0, L.list1, L.place_of, L.scan_state[1], L.sort_state, k0, k1,
                       v0, static_cast<unsigned*>(inst_rec.p), hist(), sort_state(), tile_bits, (long long)m_cap, num_sms,
                       ctl(), s);
     mark(s, 4);

@@ -736,15 +736,15 @@ int word_tile_passes(int tile_bits) { return tile_bits <= kSortBits ? 1 : (tile_
 
 void launch_sort_large(const ProjBuffers& pb, const ViewDev* views, int stride, long long n_items,
                        unsigned long long* list0, unsigned long long* list1, unsigned* place_of,
-                       unsigned long long* list_state, unsigned long long* words0, unsigned long long* words1,
-                       unsigned* vals_out, unsigned* inst_rec, unsigned* hist, unsigned* state, int tile_bits,
-                       long long m_cap, int num_sms, Control* ctl, cudaStream_t s) {
+                       unsigned long long* list_state, unsigned* depth_state, unsigned long long* words0,
+                       unsigned long long* words1, unsigned* vals_out, unsigned* inst_rec, unsigned* hist,
+                       unsigned* tile_state, int tile_bits, long long m_cap, int num_sms, Control* ctl, cudaStream_t s) {
   const unsigned rec_tiles = (unsigned)((n_items + kSortTile - 1) / kSortTile);
   const unsigned inst_tiles = (unsigned)((m_cap + kSortTile - 1) / kSortTile);
   launch_dep(k_depth_hist, dim3((unsigned)(2 * num_sms)), dim3(1024), 0, s, list0, hist, ctl);
   for (int p = 0; p < kDepthPasses; ++p)
     launch_dep(k_sort_pass_words, dim3(rec_tiles), dim3(kSortThreads), sizeof(WordSmem), s, (p & 1) ? list1 : list0,
-        (p & 1) ? list0 : list1, nullptr, 1, hist + p * kSortBins, state + (size_t)p * rec_tiles * kSortBins,
+        (p & 1) ? list0 : list1, nullptr, 1, hist + p * kSortBins, depth_state + (size_t)p * rec_tiles * kSortBins,
         32 + p * kSortBits, p, ctl, kSpinLimit);
   launch_dep(k_scan<SCAN_LIST>, dim3((unsigned)((n_items + kScanTile - 1) / kScanTile)), dim3(kScanThreads), 0, s,
       pb.count, place_of, 0ll, list_state, ctl, 0ull, nullptr, nullptr, kSpinLimit, list0, nullptr);
@@ -754,12 +754,11 @@ void launch_sort_large(const ProjBuffers& pb, const ViewDev* views, int stride, 
   // the last pass ends in words0: start in words[tp & 1]
   launch_dep(k_emit_words, dim3((unsigned)(4 * num_sms)), dim3(512), 0, s, pb, views, stride, place_of,
       (tp & 1) ? words1 : words0, inst_rec, hist + kDepthPasses * kSortBins, tp, ctl);
-  unsigned* tstate = state + (size_t)kDepthPasses * rec_tiles * kSortBins;
   for (int p = 0; p < tp; ++p) {
     const bool from1 = ((tp - p) & 1) != 0;
     launch_dep(k_sort_pass_words, dim3(inst_tiles), dim3(kSortThreads), sizeof(WordSmem), s, from1 ? words1 : words0,
         from1 ? words0 : words1, p == tp - 1 ? vals_out : nullptr, 0, hist + (kDepthPasses + p) * kSortBins,
-        tstate + (size_t)p * inst_tiles * kSortBins, 32 + p * kSortBits, kDepthPasses + p, ctl, kSpinLimit);
+        tile_state + (size_t)p * inst_tiles * kSortBins, 32 + p * kSortBits, kDepthPasses + p, ctl, kSpinLimit);
   }
 }
 
