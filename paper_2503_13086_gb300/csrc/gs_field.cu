@@ -25,13 +25,11 @@
 #include <memory>
 #include <mutex>
 #include <numeric>
-#include <thread>
 #include <unordered_map>
 #include <vector>
 
-#include <unistd.h>
-
 #include "gs_engine.h"
+#include "host_pages.h"
 
 namespace gs {
 
@@ -1047,36 +1045,12 @@ gs_status gs_field_set_gaussians(gs_field* ff, const float* host, int64_t n, int
   return GS_OK;
 }
 
-// First touch, on the host, of the rows a device copy is about to overwrite.  On Grace-Blackwell the copy
-// writes ordinary host memory directly; a page that does not exist yet is then a fault of the device, and
-// those take about 50 us per 64 KiB page: 284 ms for 354 MB of fresh memory, against 1.9 ms once the pages
-// exist.  The host makes them in 11 ms, eight threads in 3 ms.  Only bytes the copy overwrites are written
-// (the first of a row and of every page inside it); pages that exist already cost nothing to speak of.
-static void first_touch(float* dst, size_t row_bytes, size_t pitch_bytes, int rows) {
-  const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
-  const auto touch = [=](int r0, int r1) {
-    for (int r = r0; r < r1; ++r) {
-      volatile char* row = reinterpret_cast<char*>(dst) + (size_t)r * pitch_bytes;
-      const size_t to_next = page - (reinterpret_cast<uintptr_t>(row) & (page - 1));
-      row[0] = 0;
-      for (size_t o = to_next; o < row_bytes; o += page) row[o] = 0;
-    }
-  };
-  // a thread costs about as much as 50 pages
-  const size_t pages = row_bytes * (size_t)rows / page;
-  const int n = (int)std::min<size_t>({8, std::max<size_t>(1, std::thread::hardware_concurrency()), pages / 200 + 1});
-  std::vector<std::thread> threads;
-  int done = 0;
-  try {
-    for (int k = 1; k < n; ++k) {
-      const int upto = rows * k / n;
-      threads.emplace_back(touch, done, upto);
-      done = upto;
-    }
-  } catch (...) {  // no thread or no memory for one: this thread does the rest
-  }
-  touch(done, rows);
-  for (std::thread& t : threads) t.join();
+// Makes the host pages of the rows a device copy is about to overwrite (ordinary host memory only).
+static void make_host_pages(float* dst, size_t row_bytes, size_t pitch_bytes, int rows) {
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) cudaGetLastError();
+  else if (at.type != cudaMemoryTypeUnregistered) return;
+  gs::make_pages(dst, row_bytes, pitch_bytes, (size_t)rows);
 }
 
 gs_status gs_field_get_gaussians(gs_field* ff, float* host, float* host_m, float* host_v, int64_t dst_stride,
@@ -1086,14 +1060,15 @@ gs_status gs_field_get_gaussians(gs_field* ff, float* host, float* host_m, float
   if (out_n) *out_n = f->n;
   if (!host && !host_m && !host_v) return GS_OK;
   if (dst_stride < f->n) return fail(GS_ERR_INVALID_ARG, "dst_stride < n");
-  cudaStreamSynchronize(f->stream);
+  cudaError_t e = cudaStreamSynchronize(f->stream);
+  if (e != cudaSuccess) return fail(GS_ERR_CUDA, cudaGetErrorString(e));  // before anything is written
   const gs::DevBuf* src[3] = {&f->params, &f->adam_m, &f->adam_v};
   float* dst[3] = {host, host_m, host_v};
   for (int k = 0; k < 3; ++k) {
     if (!dst[k] || f->n == 0) continue;
-    first_touch(dst[k], (size_t)f->n * 4, (size_t)dst_stride * 4, gs::kNumParams);
-    cudaError_t e = cudaMemcpy2D(dst[k], (size_t)dst_stride * 4, src[k]->p, (size_t)f->stride * 4, (size_t)f->n * 4,
-                                 gs::kNumParams, cudaMemcpyDeviceToHost);
+    make_host_pages(dst[k], (size_t)f->n * 4, (size_t)dst_stride * 4, gs::kNumParams);
+    e = cudaMemcpy2D(dst[k], (size_t)dst_stride * 4, src[k]->p, (size_t)f->stride * 4, (size_t)f->n * 4, gs::kNumParams,
+                     cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, cudaGetErrorString(e));
   }
   return GS_OK;
@@ -1373,7 +1348,7 @@ gs_status gs_field_densify_stats(gs_field* ff, float* host_sum, float* host_coun
   if (e != cudaSuccess) return fail(GS_ERR_CUDA, cudaGetErrorString(e));
   const float* d = static_cast<const float*>(f->dstat.p);
   for (float* dst : {host_sum, host_count})
-    if (f->n > 0 && dst) first_touch(dst, (size_t)f->n * 4, (size_t)f->n * 4, 1);
+    if (f->n > 0 && dst) make_host_pages(dst, (size_t)f->n * 4, (size_t)f->n * 4, 1);
   if (f->n > 0 && host_sum && cudaMemcpy(host_sum, d, (size_t)f->n * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
     return fail(GS_ERR_CUDA, "reading the statistics failed");
   if (f->n > 0 && host_count &&
