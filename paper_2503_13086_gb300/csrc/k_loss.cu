@@ -172,7 +172,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
   // Directly after the blend forward (tile_done given) this grid does not wait for the forward to
   // complete: its CTAs are scheduled once every forward CTA is running (the forward is persistent,
   // so every one of them is resident and makes progress), and each block waits only for the tiles
-  // under its window.  What the forward writes (render, counters) is then read through L2.
+  // under its window.  What the forward writes (render, counters) is then read through L2.  A block that
+  // does not see its tiles or the forward's warps finish (a void step, a wait that gave up) waits for the whole
+  // forward before it leaves: the step after this one must not meet a forward that still runs.
   if (!tile_done) dep_wait();
   dep_release();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -182,6 +184,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
   // (step_void, read through L2: the blend forward may still be running and set the bit)
   if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(&ctl->error) != 0u)) {
     if (threadIdx.x == 0 && ledger) atomicOr(&ledger->error, ld_relaxed_u32(&ctl->error) & kErrTimeout);
+    if (tile_done) dep_wait();
     return;
   }
   const long long b = blockIdx.x;
@@ -200,7 +203,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
       bool ok = true;
       for (int k = threadIdx.x; k < nt && ok; k += 32)
         ok = wait_count(tile_done + V.tile_base + (long long)(ty0 + k / ntx) * V.gx + (tx0 + k % ntx), 1u, spin_limit);
-      if (!ok) atomicOr(&ctl->error, kErrTimeout);
+      if (!ok) {
+        atomicOr(&ctl->error, kErrTimeout);
+        dep_wait();
+      }
     }
     __syncthreads();
   }
@@ -371,7 +377,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
   if (threadIdx.x == 0) {
     // the forward's counters: complete once every forward warp has counted itself (when this grid
     // did not wait for the forward), read through L2
-    if (tile_done && !wait_count(&ctl->fwd_done, (unsigned)fwd_warps, spin_limit)) atomicOr(&ctl->error, kErrTimeout);
+    if (tile_done && !wait_count(&ctl->fwd_done, (unsigned)fwd_warps, spin_limit)) {
+      atomicOr(&ctl->error, kErrTimeout);
+      dep_wait();
+    }
     const unsigned long long gp_pixels = ld_relaxed_u64(&ctl->gp_pixels), blended = ld_relaxed_u64(&ctl->blended);
     const unsigned long long gp_sq = ld_relaxed_u64(&ctl->gp_sq), pairs = ld_relaxed_u64(&ctl->pairs);
     double loss = total / (double)n_views;
