@@ -985,9 +985,14 @@ void launch_backward_kernel(const ViewDev* views, int n_views, long long n_tiles
 }
 
 // A warp works on an item for 25 - 45 us (about 40 Gaussians in its two rounds, 0.6 - 1 us each), so with few
-// items the kernel lasts as long as the slowest of them: two warps share each up to eight items per pair
-// of warps on the chip.  One warp against two: 33 -> 25 us at 220 items (at most, by the buffers), 39 -> 26 at
-// 1.6k, 45 -> 43 at 3.6k, 60 -> 56 at 5.9k, 81 -> 80 at 9.0k; with 14k and more the second head per item shows.
+// items the kernel lasts as long as the slowest of them: two warps share each up to one item per pair of warps
+// on the chip, and up to eight where the lists are short (about 300 entries each, 380 of capacity).  One warp
+// against two: 33 -> 25 us at 220 items (at most, by the buffers), 39 -> 26 at 1.6k, 36 -> 33 at 2.8k (297 entries
+// per list), 45 -> 43 at 3.6k (75), 60 -> 56 at 5.9k (78), 81 -> 80 at 9.0k (84); with 14k and more the second head
+// per item shows.  In longer lists most items lie behind the depth where the pixels stop, and the second
+// head is all there is: 40 and 40 us at 3.2k items (377 per list), a whole step 271 -> 283 us at 11k (1500), and
+// with several sessions on the chip more: a round of eight sessions' steps 338 -> 387 us (30k Gaussians at 160
+// x 120) without and with sharing there.
 template <int TW, int TH, bool LOAD>
 void launch_backward_instance(const ViewDev* views, int n_views, long long n_tiles, const uint2* ranges,
                               const unsigned* vals, const ProjBuffers& pb, Control* ctl, const float* image,
@@ -996,7 +1001,8 @@ void launch_backward_instance(const ViewDev* views, int n_views, long long n_til
                               long long m_cap, int num_sms, cudaStream_t s) {
   if constexpr (TW * TH > 64 * kBwdPairs) {
     const long long items = (m_cap >> 5) + n_tiles + 1;  // at most
-    if (items <= 8ll * num_sms * bwd_occupancy<TW, TH, LOAD, true>() * (kBwdWarps / 2)) {
+    const long long per_pair = m_cap <= 380 * n_tiles ? 8 : 1;
+    if (items <= per_pair * num_sms * bwd_occupancy<TW, TH, LOAD, true>() * (kBwdWarps / 2)) {
       launch_backward_kernel<TW, TH, LOAD, true>(views, n_views, n_tiles, ranges, vals, pb, ctl, image, dimage, ckpt,
                                                  cmask, chunk_tile, tile_chunks, ginst, gp, sp, num_sms, s);
       return;
