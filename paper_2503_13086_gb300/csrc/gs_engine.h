@@ -139,7 +139,7 @@ struct Raster {
     unsigned* place_of;                 // per record: where its instances go
     unsigned long long* scan_state[2];  // look-back states of the list and of the scan of its counts
     unsigned* sort_state;               // and of the depth passes
-    size_t state_bytes;                 // of the three together (contiguous from scan_state[0], cleared by each step)
+    size_t state_bytes;                 // of the three together (contiguous from scan_state[0], cleared by K1)
   };
   LargeScratch large_scratch() const;
   bool list_built = false;  // the last forward head listed its records

@@ -44,8 +44,9 @@ struct Tiling {
 int tiling_candidates(Tiling* out, int cap);  // returns how many; fills up to cap
 bool tiling_supported(const Tiling& t);
 
+// clear (nullable): n_clear words, at most one per record, set to 0 (what the step's later kernels count on).
 void launch_project(const float* params, int stride, int n_views, const StepParams* sp, const ViewDev* views,
-                    const ProjBuffers& out, cudaStream_t s);
+                    const ProjBuffers& out, unsigned* clear, long long n_clear, cudaStream_t s);
 // K9a (per-record sums of the instance gradients, into g2s: 9 planes of views x stride floats) and
 // K9 + K10.
 void launch_project_backward(float* params, int stride, int n_views, const StepParams* sp, const ViewDev* views,

@@ -181,16 +181,23 @@ Raster::LargeScratch Raster::large_scratch() const {
   const size_t recs = (size_t)n_views * stride;  // a multiple of 32
   const size_t scan_tiles = (recs + kScanTile - 1) / kScanTile, sort_tiles = (recs + kSortTile - 1) / kSortTile;
   static_assert(kDepthPasses * kSortBins * 4 <= kSortTile, "at most a byte per record and a last tile's");
-  static_assert(22 * kLargeRecords + kSortTile + 16 <= 36 * kLargeRecords, "the lists' 20 bytes and the states fit g2s");
+  static_assert(22 * kLargeRecords + kSortTile + 3 * 512 <= 36 * kLargeRecords, "the lists' 20 bytes and the states fit g2s");
+  // every part starts on a 256-byte boundary: a warp reads 32 neighbouring words of a look-back state at a time
+  // (off the boundary K4 took 290 instead of 285 us at 3M records)
+  const auto whole = [](size_t bytes) { return (bytes + 255) & ~size_t(255); };
   LargeScratch L;
-  char* base = static_cast<char*>(g2s.p);
-  L.list0 = reinterpret_cast<unsigned long long*>(base);
-  L.list1 = L.list0 + recs;
-  L.place_of = reinterpret_cast<unsigned*>(L.list1 + recs);
-  L.scan_state[0] = reinterpret_cast<unsigned long long*>(L.place_of + recs);
-  L.scan_state[1] = L.scan_state[0] + scan_tiles;
-  L.sort_state = reinterpret_cast<unsigned*>(L.scan_state[1] + scan_tiles);
-  L.state_bytes = 2 * scan_tiles * 8 + (size_t)kDepthPasses * sort_tiles * kSortBins * 4;
+  char* at = static_cast<char*>(g2s.p);
+  const auto take = [&](size_t bytes) {
+    char* p = at;
+    at += whole(bytes);
+    return p;
+  };
+  L.list0 = reinterpret_cast<unsigned long long*>(take(recs * 8));
+  L.list1 = reinterpret_cast<unsigned long long*>(take(recs * 8));
+  L.place_of = reinterpret_cast<unsigned*>(take(recs * 4));
+  for (auto& state : L.scan_state) state = reinterpret_cast<unsigned long long*>(take(scan_tiles * 8));
+  L.sort_state = reinterpret_cast<unsigned*>(take((size_t)kDepthPasses * sort_tiles * kSortBins * 4));
+  L.state_bytes = (size_t)(at - reinterpret_cast<char*>(L.scan_state[0]));
   return L;
 }
 unsigned* Raster::hist() const { return reinterpret_cast<unsigned*>(zeroB.p); }
@@ -361,9 +368,9 @@ gs_status Raster::enqueue_forward_head(cudaStream_t s, const float* params, int 
   if (!size_exactly) cudaMemsetAsync(zeroB.p, 0, zeroB_bytes, s);
   list_built = large();
   const LargeScratch L = list_built ? large_scratch() : LargeScratch{};
-  if (list_built) cudaMemsetAsync(L.scan_state[0], 0, L.state_bytes, s);
   mark(s, 0);
-  launch_project(params, stride_, n_views, sp(), vd(), proj(), s);
+  launch_project(params, stride_, n_views, sp(), vd(), proj(), reinterpret_cast<unsigned*>(L.scan_state[0]),
+                 (long long)(L.state_bytes / 4), s);
   mark(s, 1);
   const long long n_items = (long long)n_views * stride_;
   launch_scan(proj().count, proj().offsets, n_items, scan_state(), ctl(), size_exactly ? ~0ull : m_cap, ledger(), s,

@@ -185,9 +185,14 @@ __device__ __forceinline__ bool geo_forward(const ViewDev& V, const float mu[3],
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128, 8) k_project(const float* __restrict__ params, int stride,
                                                  const StepParams* __restrict__ sp,
-                                                 const ViewDev* __restrict__ views, int n_views, ProjBuffers out) {
+                                                 const ViewDev* __restrict__ views, int n_views, ProjBuffers out,
+                                                 unsigned* __restrict__ clear, long long n_clear) {
   dep_wait();
   dep_release();
+  if (clear) {  // the look-back states of a large step (at most a word per record)
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n_clear) clear[k] = 0u;
+  }
   const int v = (int)(blockIdx.x % (unsigned)n_views);
   const int i = (int)(blockIdx.x / (unsigned)n_views * blockDim.x + threadIdx.x);
   if (i >= stride) return;
@@ -1039,9 +1044,9 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ params, const 
 }
 
 void launch_project(const float* params, int stride, int n_views, const StepParams* sp, const ViewDev* views,
-                    const ProjBuffers& out, cudaStream_t s) {
+                    const ProjBuffers& out, unsigned* clear, long long n_clear, cudaStream_t s) {
   const dim3 grid((unsigned)((stride + 127) / 128) * (unsigned)n_views);
-  launch_dep(k_project, grid, dim3(128), 0, s, params, stride, sp, views, n_views, out);
+  launch_dep(k_project, grid, dim3(128), 0, s, params, stride, sp, views, n_views, out, clear, n_clear);
 }
 
 void launch_project_backward(float* params, int stride, int n_views, const StepParams* sp, const ViewDev* views,
