@@ -162,8 +162,8 @@ Raster::Raster() {
 
 Raster::~Raster() {
   DevBuf* all[] = {&sp_d, &views_d, &ledger_d, &zeroA, &zeroB, &xyo, &conic, &rgb, &depth, &radius, &rect, &count, &offsets,
-                   &clamp, &g2s, &keys0, &keys1, &vals0, &vals1, &ginst, &inst_rec, &carry, &ckpt, &cmask, &order, &tile_chunks, &partials, &block_sums, &own_image,
-                   &own_last, &own_dimage};
+                   &clamp, &g2s, &keys0, &keys1, &vals0, &vals1, &ginst, &inst_rec, &carry, &ckpt, &cmask, &order, &tile_chunks,
+                   &partials, &block_sums, &own_image, &own_last, &own_dimage};
   for (DevBuf* b : all) b->release(&bytes_in_use);
   if (sp_h) cudaFreeHost(sp_h);
   if (views_h) cudaFreeHost(views_h);
@@ -285,7 +285,8 @@ gs_status Raster::ensure_records(int stride_) {
   const long long scan_tiles = (recs + kScanTile - 1) / kScanTile;
   if ((s = zeroA.reserve(kCtlBytes + scan_tiles * 8, &bytes_in_use))) return s;
   zeroA_bytes = kCtlBytes + scan_tiles * 8;
-  if ((s = partials.reserve(n_pix * 10 * 4, &bytes_in_use)) || (s = block_sums.reserve(n_loss_blocks * 16 * (n_loss_blocks <= loss_split_blocks(num_sms) ? 3 : 1), &bytes_in_use)))
+  const long long loss_ctas = n_loss_blocks * (n_loss_blocks <= loss_split_blocks(num_sms) ? 3 : 1);
+  if ((s = partials.reserve(n_pix * 10 * 4, &bytes_in_use)) || (s = block_sums.reserve(loss_ctas * 16, &bytes_in_use)))
     return s;
   return GS_OK;
 }

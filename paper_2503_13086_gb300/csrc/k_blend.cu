@@ -14,8 +14,8 @@
 // walked in chunks of 32.  A warp skips a Gaussian outright when the bounding box of its 1/255 cutoff
 // ellipse misses the warp's block (warp-uniform).  The others are taken two at a time (four when the tiles
 // are few, see few_tiles) without a branch: every lane evaluates their exponents and alphas, then blends
-// them in list order under predicates.  A pixel's walk is one dependent chain, and the longest lists set the kernel's duration from a few
-// thousand Gaussians up, so what counts is the chain's length per candidate: with a branch per test
+// them in list order under predicates.  A pixel's walk is one dependent chain, and the longest lists set
+// the kernel's duration from a few thousand Gaussians up, so what counts is the chain's length per candidate: with a branch per test
 // (cutoff, alpha, stop) it was about 300 cycles, in this form about 210 when a CTA has its SM to itself,
 // and about 48 instead of 62 instructions.  A stopped pixel's x becomes NaN, which fails every later
 // test by itself; the last index and G_p follow from the chunk's mask.  Measured: 54 -> 32 us on a
@@ -47,7 +47,7 @@
 // is written once, to its own slot.  K8 is bound by issue (66 % at 16 warps per SM; 240 instructions per
 // Gaussian and round, of which 1.4 pair bodies are about 95) and, with few items, by one warp's latency
 // (5 cycles per instruction).  The load term is a template flag (its test and weights cost 4 registers
-// and an instruction per pair), the reciprocal of 1 - alpha the bare instruction, the conic terms' factors
+// and an instruction per pair), the reciprocal of 1 - alpha is rcp.approx.ftz, the conic terms' factors
 // are applied once per row sum, and the tile's position takes 32-bit divisions: 1269 -> 1221 us for nine
 // views of 500k Gaussians, 152 -> 144 at 1297 x 840 (200k), 48 -> 45 at 640 x 361 (20k), the same bits.
 // Measured and not kept: the records held twice in shared memory for the packed operands (16 bytes more
@@ -128,12 +128,12 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint2* __restrict__ r
 // Work flows through the CTA as jobs: a job is one staged batch (up to BATCH sorted entries) of one
 // tile, and kFwdBufs jobs are in shared memory at a time.  Each warp walks every job in order (its 8 x 4
 // block of the job's tile); the warp that finishes job j first stages job j + 1 into the other
-// buffer of job j + 1 - kFwdBufs once every warp is through that job -- the next batch of the same tile while any warp of it still blends, else the first batch
-// of the next tile in the longest-first order -- so staging overlaps the slower warps' walk and a
+// buffer of job j + 1 - kFwdBufs once every warp is through that job -- the next batch of the same tile while
+// any warp of it still blends, else the first batch of the next tile in the longest-first order -- so staging overlaps the slower warps' walk and a
 // warp waits only when it has caught up with the staging, not for the tile's slowest block.  A job
 // is published by an mbarrier (`full`, 32 arrivals: the staging warp's lanes) and released by
 // another (`empty`, one arrival per warp).  Every wait is bounded: a wait that gives up sets
-// kErrTimeout and its warp leaves (the host reports GS_ERR_TIMEOUT; the outputs are then unspecified).
+// kErrTimeout and its warp leaves (the host reports GS_ERR_TIMEOUT; the image is then unspecified).
 namespace {
 constexpr int kFwdBufs = 2;  // jobs in shared memory at a time (3 measured 112 against 107 us)
 
@@ -590,9 +590,13 @@ void init_forward_instance() {
 // 150k Gaussians (48 tiles), 110 -> 84 at 160 x 120 of 30k (80), 164 -> 133 at 300 x 200 of 120k (247), 32 -> 26
 // at 128 x 97 of 3k, 70 -> 57 at 640 x 360 of 60k (920), 61 -> 62 at 960 x 540 of 60k (2040), 91 -> 75 at
 // 1000 x 600 of 200k (2394).  Smaller tiles have shorter lists for the same count and stay under the line
-// only on smaller images.  With 4346 tiles it depends on the lists, which the host does not know (262 against 330 us at 1.9M, but 123 against
-// 110 at 200k with large Gaussians over the image), and with 8160 and more the lost occupancy shows (148
-// against 118, 1042 against 751 on nine views).  Eight per round: 471 us on the 48 tiles.
+// only on smaller images.  With 4346 tiles it depends on the lists, which the host does not know (262 against
+// 330 us at 1.9M, but 123 against 110 at 200k with large Gaussians over the image), and with 8160 and more
+// the lost occupancy shows (148 against 118, 1042 against 751 on nine views).  Eight per round: 471 us on the
+// 48 tiles.  Several sessions on one GPU give part of it back: whole steps of one session, ring scenes of 120k
+// to 500k Gaussians at 300 x 200 to 640 x 360, take 394 -> 353 down to 624 -> 587 us, a round of eight sessions'
+// steps 931 -> 917 and 2911 -> 2906; but where every list is as long as the next (a cube of 120k in the same
+// 300 x 200) 284 -> 284 us alone and 1188 -> 1273 by eight.
 bool few_tiles(long long n_tiles, int num_sms) { return n_tiles <= 16ll * num_sms; }
 
 // Persistent grid of one K6 instance: every resident CTA, at most one per tile.
@@ -664,7 +668,8 @@ long long forward_warps(const Tiling& tl, long long n_tiles, int num_sms) {
 // ---------------------------------------------------------------------------------------------
 // K8
 // ---------------------------------------------------------------------------------------------
-// 1 / x for x in [1 - kAlphaMax, 1] (no range scaling needed; within 1 ulp).
+// 1 / x for x in [1 - kAlphaMax, 1]: rcp.approx.ftz is within 1 ulp, and neither x nor 1 / x is near the
+// denormal range.
 __device__ __forceinline__ float fast_rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -749,7 +754,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) k_blend_backward(
     const int cnt = min(kChunk, L - base);
     const int v = view_of_tile(views, n_views, t);
     const ViewDev& V = views[v];
-    const int local = (int)(t - V.tile_base);  // (32-bit: a 64-bit division is a subroutine)
+    const int local = (int)(t - V.tile_base);
     const int tx = local % V.gx, ty = local / V.gx;
     const long long cid = id;
 
