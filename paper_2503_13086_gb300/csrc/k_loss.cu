@@ -183,12 +183,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
   LossFwdSmem& S = *reinterpret_cast<LossFwdSmem*>(smem_raw);
   __shared__ double s_red[2][8];
   __shared__ bool s_last;
-  // (step_void, read through L2: the blend forward may still be running and set the bit)
-  if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(&ctl->error) != 0u)) {
-    if (threadIdx.x == 0 && ledger) atomicOr(&ledger->error, ld_relaxed_u32(&ctl->error) & kErrTimeout);
-    if (tile_done) dep_wait();
-    return;
-  }
   const long long b = blockIdx.x;
   const int v = view_of_block(views, n_views, b);
   const ViewDev& V = views[v];
@@ -196,25 +190,35 @@ __global__ void __launch_bounds__(kThreads, 3) k_loss_forward(const ViewDev* __r
   const long long lb = b - V.loss_block_base;
   const int bx = (int)(lb % bxn), by = (int)(lb / bxn);
   const int ox = bx * kBX, oy = by * kBY;
+  bool none = !tile_done && step_void(ctl);
   if (tile_done) {
     if (threadIdx.x < 32) {
-      // the tiles under the staged window (clipped to the image), one lane per tile
-      const int tx0 = max(0, ox - kR) / V.tw, tx1 = min(V.W - 1, ox + kBX + kR - 1) / V.tw;
-      const int ty0 = max(0, oy - kR) / V.th, ty1 = min(V.H - 1, oy + kBY + kR - 1) / V.th;
-      const int ntx = tx1 - tx0 + 1, nt = ntx * (ty1 - ty0 + 1);
-      bool ok = true;
-      for (int k = threadIdx.x; k < nt && ok; k += 32)
-        ok = wait_count(tile_done + V.tile_base + (long long)(ty0 + k / ntx) * V.gx + (tx0 + k % ntx), 1u, spin_limit);
-      if (!ok) {
-        atomicOr(&ctl->error, kErrTimeout);
-        dep_wait();
+      // the blend forward may still be running and set the error bit: read through L2, by one warp for the block
+      none = ld_relaxed_u32(&ctl->error) != 0u;
+      if (!__any_sync(0xffffffffu, none)) {
+        // the tiles under the staged window (clipped to the image), one lane per tile
+        const int tx0 = max(0, ox - kR) / V.tw, tx1 = min(V.W - 1, ox + kBX + kR - 1) / V.tw;
+        const int ty0 = max(0, oy - kR) / V.th, ty1 = min(V.H - 1, oy + kBY + kR - 1) / V.th;
+        const int ntx = tx1 - tx0 + 1, nt = ntx * (ty1 - ty0 + 1);
+        bool ok = true;
+        for (int k = threadIdx.x; k < nt && ok; k += 32)
+          ok = wait_count(tile_done + V.tile_base + (long long)(ty0 + k / ntx) * V.gx + (tx0 + k % ntx), 1u, spin_limit);
+        if (!ok) {
+          atomicOr(&ctl->error, kErrTimeout);
+          dep_wait();
+        }
       }
     }
-    __syncthreads();
+    none = __syncthreads_or(none);
     // Only now may the loss backward's CTAs come: released at the start, they sat on the SMs (53 KB of shared
     // memory each) through the whole blend forward, where other sessions' steps could have run (a round of four
     // sessions' steps, 120k Gaussians at 300 x 200: 668 us, so 646; one session's 283 either way).
-    dep_release();
+    if (!none) dep_release();
+  }
+  if (none) {
+    if (threadIdx.x == 0 && ledger) atomicOr(&ledger->error, ld_relaxed_u32(&ctl->error) & kErrTimeout);
+    if (tile_done) dep_wait();
+    return;
   }
   const long long HW = (long long)V.W * V.H;
   const float* X = image + 3 * V.pix_base;
