@@ -207,8 +207,8 @@ def roofline(kernel_ms, steps, st, n, passes, peaks, peaks_kind, traffic, n_sms=
 # summaries of the current kernels (profiles/), taken with the tiling below; None for a kernel
 # changed since its capture.
 TRAFFIC_TILING = (16, 16, 256)
-TRAFFIC = {"K8 blend bwd": 62.5e6, "K6 blend fwd": 21.7e6, "K9+K10 project bwd + Adam": 253.5e6,
-           "K4 sort": 5 * 4.1e6, "K7 loss": 94.3e6}
+TRAFFIC = {"K8 blend bwd": 62.9e6, "K6 blend fwd": 22.5e6, "K9+K10 project bwd + Adam": 256.7e6,
+           "K4 sort": 5 * 4.1e6, "K7 loss": 94.5e6, "K1 project": 47.5e6}
 
 
 def cpu_baseline_run(steps, warmup, seed=0, rows=None):
